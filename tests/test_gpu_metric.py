@@ -51,3 +51,24 @@ def test_local_metric_gaussian_mixture():
     ref = oracle.local_metric(model, None, th, 0.8)
     M = ctx.local_metric(G.to_dev(th), 0.8)["mass"].cpu().numpy()
     assert np.allclose(M, ref, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("name", ["tiny", "bbh11"])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 65])
+def test_local_metric_block_edges(name, n):
+    """A CTA holds 32 particles: counts around its edge give, row by row, the matrices of the same particles in a
+    larger call (bit for bit), each output asked for alone too, and no row past the last is written."""
+    G.require_gpu()
+    w = inputs.WORKLOADS[name]()
+    ev, ctx, th_inj, _ = G.event_pair(w, seed=0)
+    th = G.to_dev(np.concatenate([inputs.prior_draws(w, 40, 7), inputs.ball(w, th_inj, 40, 8, rel=1e-3)]))
+    full = ctx.local_metric(th, 0.6)
+    ref = oracle.local_metric(helpers.oracle_model(w), ev, th[:n].cpu().numpy(), 0.6)
+    assert np.max(_scaled_err(full["mass"][:n].cpu().numpy(), ref)) < 1e-8
+    for want in (("mass",), ("inv_mass",), ("chol",), ("mass", "inv_mass", "chol")):
+        part = ctx.local_metric(th[:n].contiguous(), 0.6, want=want)
+        for k in want:
+            assert torch.equal(part[k], full[k][:n]), (k, want)
+    guard = torch.full((n + 1, w.n_dim, w.n_dim), -7.0, dtype=torch.float64, device="cuda")
+    rc = api.lib().sharpy_local_metric(ctx._h, n, api._ptr(th), 0.6, None, api._ptr(guard), None, api._stream())
+    assert rc == 0 and torch.equal(guard[:n], full["inv_mass"][:n]) and bool((guard[n] == -7.0).all())
