@@ -70,7 +70,7 @@ WORK = {p: work(p) for p in ("mixed", "split", "fp64")}
 # Each kernel's counts are keyed to the device-code files its instructions
 # come from (context.cuh, the host-side context, is not among them).
 COUNTED_SOURCES = {"nuts": ["nuts_kernel.cuh", "sweep.cuh", "physics.cuh", "common.cuh", "dfloat.cuh"],
-                   "loglike": ["loglike_kernel.cuh", "split_stage.cuh", "bulk.cuh", "sweep.cuh", "physics.cuh",
+                   "loglike": ["loglike_kernel.cuh", "bulk.cuh", "sweep.cuh", "physics.cuh",
                                "common.cuh", "dfloat.cuh"]}
 COUNTED = {"sources_sha256_16": {"nuts": "4c9bc0a722a82040", "loglike": "43066a7c70b78fc5"},
            "nuts": {"mixed": {"fp64": 2.9620, "fp32": 107.01},

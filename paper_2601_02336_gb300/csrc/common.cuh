@@ -28,27 +28,28 @@ __host__ __device__ constexpr int large_pn(int i) { return i < 3 ? i : 4; }
 __host__ __device__ constexpr int small_pn(int i) { return i == 0 ? 3 : i + 4; }
 __host__ __device__ constexpr bool is_large_pn(int j) { return j < 3 || j == 4; }
 
-// Staged tables of a long segment (K >= kStageMinBins): one contiguous record
-// per block of kStageBins bins, so that one bulk copy brings a block's tables
-// into shared memory. Record layout (bins g kStageBins + i, i < kStageBins;
-// zeros past the last bin):
-//   float  b32[9][kStageBins]       basis functions, FP32 hi parts
-//   float  lo[5][kStageBins]        FP32 lo parts of x, y, y ln f, y^2 and f
-//   double b64[4][kStageBins]       x^5, x^3, x^2, ln f in FP64
-//   float2 e32[n_det][kStageBins]   pre-whitened data
-// Every offset and the record size are multiples of 16 bytes.
+// Tables of the mixed and split sweeps: tiles of kTileBins bins, a tile's quads
+// (16 bytes a bin) one after the other, so that a warp (lane = bin) reads each
+// quad with one 16-byte load a lane at a constant offset: 7 loads a bin for the
+// mixed sweep and 6 for the split one, where separate arrays took 21 and 24
+// with an address each. Zeros past the last bin.
+//   mixed: 0 B hi {3, 6, 5, 7}   1 B hi {0, 1, 2, 4}   2 B lo {3, 6, 5, 7}
+//          3 {f hi, f lo, E_0}   4 {E_1, E_2}          5, 6 B {0, 1}, {2, 4} in FP64
+//   split: 0 B hi {0, 2, 1, 3}   1 B hi {4, 6, 5, 7}   2, 3 their lo parts
+//          4 {f hi, f lo, E_0}   5 {E_1, E_2}
+// (the orders put the terms of a pairwise sum into the same halves of two
+// register pairs). A block of kStageBins bins is contiguous: one bulk copy
+// brings it into shared memory (the staged kernel of long segments).
+constexpr int kTileBins = 32;
 constexpr int kStageBins = 256;
 constexpr int64_t kStageMinBins = 65536;
-__host__ __device__ constexpr int stage_off_lo() { return kNBasis * kStageBins * 4; }
-__host__ __device__ constexpr int stage_off_b64() { return stage_off_lo() + 5 * kStageBins * 4; }
-__host__ __device__ constexpr int stage_off_e32() { return stage_off_b64() + 4 * kStageBins * 8; }
-__host__ __device__ constexpr int stage_rec_bytes(int n_det) { return stage_off_e32() + n_det * kStageBins * 8; }
-// row of basis function j among the staged lo parts (j = 3, 5, 6, 7, 8) and FP64 rows (j = 0, 1, 2, 4)
-__host__ __device__ constexpr int stage_lo_row(int j) { return j == 3 ? 0 : j == 5 ? 1 : j == 6 ? 2 : j == 7 ? 3 : 4; }
-__host__ __device__ constexpr int stage_b64_row(int j) { return j == 4 ? 3 : j; }
-static_assert(stage_off_lo() % 16 == 0 && stage_off_b64() % 16 == 0 && stage_off_e32() % 16 == 0 &&
-                  stage_rec_bytes(1) % 16 == 0,
-              "bulk copies move multiples of 16 bytes between 16-byte aligned addresses");
+__host__ __device__ constexpr int tile_basis(bool split, int i) {  // basis function of hi word i < 8
+  return split ? (i == 0 ? 0 : i == 1 ? 2 : i == 2 ? 1 : i == 3 ? 3 : i == 4 ? 4 : i == 5 ? 6 : i == 6 ? 5 : 7)
+               : (i == 0 ? 3 : i == 1 ? 6 : i == 2 ? 5 : i == 3 ? 7 : i < 7 ? i - 4 : 4);
+}
+__host__ __device__ constexpr int tile_quads(bool split) { return split ? 6 : 7; }
+__host__ __device__ constexpr int tile_quad_f(bool split) { return split ? 4 : 3; }
+__host__ __device__ constexpr int stage_bytes(bool split) { return kStageBins * tile_quads(split) * 16; }
 
 // Model configuration as passed to kernels (by value).
 struct DevModel {
@@ -85,15 +86,12 @@ struct DevEvent {
   float ddh_hi, ddh_lo;      // -<d|d>/2 as a double-float: hi = (float)x, lo = (float)(x - hi)
   const double* f;           // [K] f_k
   const double* b64;         // [kNBasis][K] basis functions (FP64)
-  const float* b32;          // [kNBasis][K] basis functions (FP32, = hi part)
-  const float* b32lo;        // [kNBasis][K] B - (double)hi (FP32 lo part)
   const double2* e64;        // [n_det][K] E = w conj(d) f^-7/6 (FP64)
-  const float2* e32;         // [n_det][K] same, FP32
+  const float4* tile_mixed;  // tiles of the mixed and the split sweep, whole blocks of kStageBins
+  const float4* tile_split;
   const double* pref;        // [n_det][K] prefix sums of w f^-7/3
   const double* p1;          // [n_det][kNBasis][K] prefix sums of w f^-7/3 B_m (Fisher), or null
   const double* p2;          // [n_det][kNBasis (kNBasis + 1) / 2][K] ... B_m B_n, m <= n, or null
-  const unsigned char* stage;  // staged records (see stage_rec_bytes), or null for K < kStageMinBins
-  int stage_blocks;            // records: ceil(K / kStageBins)
   DevDetector det[kMaxDet];
 };
 

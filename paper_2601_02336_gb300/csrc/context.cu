@@ -5,7 +5,6 @@
 #include <vector>
 
 #include "context.cuh"
-#include "split_stage.cuh"
 
 using namespace sharpy;
 
@@ -30,34 +29,43 @@ int check_ctx(sharpy_ctx* ctx, bool need_data) {
   return SHARPY_OK;
 }
 
-// One CTA per staged record: thread i copies bin g kStageBins + i of every
-// table the mixed sweep reads into record g of the mixed set, and of every
-// table the split sweep reads into record g of the split set (zeros past the
-// last bin).
-__global__ void stage_tables_kernel(DevEvent ev, int nb, unsigned char* out) {
-  const int g = blockIdx.x, i = threadIdx.x;
-  const int64_t K = ev.n_bins, k = (int64_t)g * kStageBins + i;
+// One CTA per block of kStageBins bins, one thread per bin: writes the bin's
+// quads of the mixed and of the split sweep's tiles.
+__global__ void __launch_bounds__(kStageBins) tile_kernel(DevEvent ev, float4* mixed, float4* split) {
+  const int64_t K = ev.n_bins, k = (int64_t)blockIdx.x * kStageBins + threadIdx.x;
   const bool in = k < K;
-  unsigned char* rec = out + (size_t)g * stage_rec_bytes(ev.n_det);
-  float* b32 = reinterpret_cast<float*>(rec);
-  float* lo = reinterpret_cast<float*>(rec + stage_off_lo());
-  double* b64 = reinterpret_cast<double*>(rec + stage_off_b64());
-  float2* e32 = reinterpret_cast<float2*>(rec + stage_off_e32());
-  for (int j = 0; j < kNBasis; ++j) b32[j * kStageBins + i] = in ? ev.b32[j * K + k] : 0.0f;
-  constexpr int lo_j[5] = {3, 5, 6, 7, 8};
-  for (int r = 0; r < 5; ++r) lo[r * kStageBins + i] = in ? ev.b32lo[lo_j[r] * K + k] : 0.0f;
-  constexpr int b64_j[4] = {0, 1, 2, 4};
-  for (int r = 0; r < 4; ++r) b64[r * kStageBins + i] = in ? ev.b64[b64_j[r] * K + k] : 0.0;
-  for (int a = 0; a < ev.n_det; ++a) e32[a * kStageBins + i] = in ? ev.e32[a * K + k] : make_float2(0.0f, 0.0f);
-  unsigned char* srec = out + split_set_offset(nb, ev.n_det) + (size_t)g * split_rec_bytes(ev.n_det);
-  float* sb32 = reinterpret_cast<float*>(srec);
-  float* slo = reinterpret_cast<float*>(srec + split_off_lo());
-  float2* se32 = reinterpret_cast<float2*>(srec + split_off_e32());
+  double b[kNBasis];
+  float hi[kNBasis], lo[kNBasis];
+  float2 E[3];
   for (int j = 0; j < kNBasis; ++j) {
-    sb32[j * kStageBins + i] = in ? ev.b32[j * K + k] : 0.0f;
-    slo[j * kStageBins + i] = in ? ev.b32lo[j * K + k] : 0.0f;
+    b[j] = in ? ev.b64[j * K + k] : 0.0;
+    hi[j] = (float)b[j];
+    lo[j] = (float)(b[j] - (double)hi[j]);
   }
-  for (int a = 0; a < ev.n_det; ++a) se32[a * kStageBins + i] = in ? ev.e32[a * K + k] : make_float2(0.0f, 0.0f);
+  for (int a = 0; a < 3; ++a) {
+    const double2 e = in && a < ev.n_det ? ev.e64[a * K + k] : make_double2(0.0, 0.0);
+    E[a] = make_float2((float)e.x, (float)e.y);
+  }
+  auto words = [&](bool sp, const float* t, int i) {
+    return make_float4(t[tile_basis(sp, i)], t[tile_basis(sp, i + 1)], t[tile_basis(sp, i + 2)], t[tile_basis(sp, i + 3)]);
+  };
+  const int64_t tile = k / kTileBins;
+  const int lane = (int)(k % kTileBins);
+  float4* m = mixed + tile * tile_quads(false) * kTileBins + lane;
+  m[0 * kTileBins] = words(false, hi, 0);
+  m[1 * kTileBins] = words(false, hi, 4);
+  m[2 * kTileBins] = words(false, lo, 0);
+  m[3 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
+  m[4 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
+  for (int i = 0; i < 2; ++i)
+    reinterpret_cast<double2*>(m)[(5 + i) * kTileBins] = make_double2(b[large_pn(2 * i)], b[large_pn(2 * i + 1)]);
+  float4* s = split + tile * tile_quads(true) * kTileBins + lane;
+  s[0 * kTileBins] = words(true, hi, 0);
+  s[1 * kTileBins] = words(true, hi, 4);
+  s[2 * kTileBins] = words(true, lo, 0);
+  s[3 * kTileBins] = words(true, lo, 4);
+  s[4 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
+  s[5 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
 }
 
 }  // namespace sharpy
@@ -65,24 +73,16 @@ __global__ void stage_tables_kernel(DevEvent ev, int nb, unsigned char* out) {
 static void free_event(sharpy_ctx* c) {
   cudaFree(c->d_f);
   cudaFree(c->d_b64);
-  cudaFree(c->d_b32);
-  cudaFree(c->d_b32lo);
   cudaFree(c->d_e64);
-  cudaFree(c->d_e32);
   cudaFree(c->d_pref);
   cudaFree(c->d_p1);
   cudaFree(c->d_p2);
-  cudaFree(c->d_stage);
-  c->d_stage = nullptr;
-  c->ev.stage = nullptr;
-  c->ev.stage_blocks = 0;
+  cudaFree(c->d_tile);
+  c->d_tile = nullptr;
   c->d_p1 = c->d_p2 = nullptr;
   c->ev.p1 = c->ev.p2 = nullptr;
   c->d_f = c->d_b64 = c->d_pref = nullptr;
-  c->d_b32 = nullptr;
-  c->d_b32lo = nullptr;
   c->d_e64 = nullptr;
-  c->d_e32 = nullptr;
   c->has_data = false;
 }
 
@@ -205,40 +205,32 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   // (K, f_min, df): a new event on the same grid and detector count keeps
   // them and the device buffers, and only the data-dependent tables are
   // rebuilt and copied.
+  const int64_t blocks = (K + kStageBins - 1) / kStageBins;
   const bool same_grid = c->has_data && c->ev.n_det == n_det && c->ev.n_bins == K && c->ev.f_min == f_min &&
                          c->ev.df == df && (int64_t)c->h_amp.size() == K;
   if (!same_grid) {
     std::vector<double> f(K), b64(kNBasis * K), amp(K);
-    std::vector<float> b32(kNBasis * K), b32lo(kNBasis * K);
     for (int64_t k = 0; k < K; ++k) {
       double fk = f_min + (double)k * df;
       f[k] = fk;
       double x = std::cbrt(1.0 / fk), y = std::cbrt(fk), l = std::log(fk);
       double x2 = x * x;
       double B[kNBasis] = {x2 * x2 * x, x2 * x, x2, x, l, y, y * l, y * y, fk};
-      for (int j = 0; j < kNBasis; ++j) {
-        b64[j * K + k] = B[j];
-        b32[j * K + k] = (float)B[j];
-        b32lo[j * K + k] = (float)(B[j] - (double)b32[j * K + k]);
-      }
+      for (int j = 0; j < kNBasis; ++j) b64[j * K + k] = B[j];
       amp[k] = std::pow(fk, -7.0 / 6.0);
     }
     free_event(c);
     bool ok = cudaMalloc(&c->d_f, K * sizeof(double)) == cudaSuccess &&
               cudaMalloc(&c->d_b64, kNBasis * K * sizeof(double)) == cudaSuccess &&
-              cudaMalloc(&c->d_b32, kNBasis * K * sizeof(float)) == cudaSuccess &&
-              cudaMalloc(&c->d_b32lo, kNBasis * K * sizeof(float)) == cudaSuccess &&
               cudaMalloc(&c->d_e64, n_det * K * sizeof(double2)) == cudaSuccess &&
-              cudaMalloc(&c->d_e32, n_det * K * sizeof(float2)) == cudaSuccess &&
+              cudaMalloc(&c->d_tile, (size_t)blocks * (stage_bytes(false) + stage_bytes(true))) == cudaSuccess &&
               cudaMalloc(&c->d_pref, n_det * K * sizeof(double)) == cudaSuccess;
     if (!ok) {
       free_event(c);
       return SHARPY_ENOMEM;
     }
     ok = cudaMemcpy(c->d_f, f.data(), K * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemcpy(c->d_b64, b64.data(), b64.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemcpy(c->d_b32, b32.data(), b32.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
-         cudaMemcpy(c->d_b32lo, b32lo.data(), b32lo.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+         cudaMemcpy(c->d_b64, b64.data(), b64.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) {
       free_event(c);
       return SHARPY_ECUDA;
@@ -252,7 +244,6 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   }
   const std::vector<double>& amp = c->h_amp;
   std::vector<double> e64(2 * n_det * K), pref(n_det * K), wamp2(n_det * K);
-  std::vector<float> e32(2 * n_det * K);
   // <d|d> with a compensated sum; P_a prefix sums of w f^-7/3 (compensated).
   double dd = 0.0, ddc = 0.0;
   for (int a = 0; a < n_det; ++a) {
@@ -264,8 +255,6 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
       // E = w conj(d) f^-7/6
       e64[2 * i] = w * dr * amp[k];
       e64[2 * i + 1] = -w * di * amp[k];
-      e32[2 * i] = (float)e64[2 * i];
-      e32[2 * i + 1] = (float)e64[2 * i + 1];
       double term = w * amp[k] * amp[k];
       wamp2[i] = term;
       double t = s + term;
@@ -279,7 +268,6 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
     }
   }
   const bool ok = cudaMemcpy(c->d_e64, e64.data(), e64.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  cudaMemcpy(c->d_e32, e32.data(), e32.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
                   cudaMemcpy(c->d_pref, pref.data(), pref.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
   if (!ok) {
     free_event(c);
@@ -306,34 +294,20 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   }
   ev.f = c->d_f;
   ev.b64 = c->d_b64;
-  ev.b32 = c->d_b32;
-  ev.b32lo = c->d_b32lo;
   ev.e64 = c->d_e64;
-  ev.e32 = c->d_e32;
   ev.pref = c->d_pref;
   ev.p1 = c->d_p1;
   ev.p2 = c->d_p2;
   for (int a = 0; a < n_det; ++a) detector_geometry(det[a], ev.det[a]);
-  // staged records of a long segment (rebuilt with every data set: they hold E)
-  if (c->model.model == SHARPY_MODEL_TAYLORF2 && K >= kStageMinBins) {
-    const int nb = (int)((K + kStageBins - 1) / kStageBins);
-    const size_t bytes = split_set_offset(nb, n_det) + (size_t)nb * split_rec_bytes(n_det);
-    if (!c->d_stage && cudaMalloc(&c->d_stage, bytes) != cudaSuccess) {
-      c->d_stage = nullptr;
-      free_event(c);
-      return SHARPY_ENOMEM;
-    }
-    stage_tables_kernel<<<nb, kStageBins>>>(ev, nb, c->d_stage);
-    if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
-      free_event(c);
-      return SHARPY_ECUDA;
-    }
-    ev.stage = c->d_stage;
-    ev.stage_blocks = nb;
-  } else {
-    ev.stage = nullptr;
-    ev.stage_blocks = 0;
+  // the sweeps' tiles (rebuilt with every data set: they hold E)
+  float4* split = c->d_tile + blocks * (stage_bytes(false) / 16);
+  tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, c->d_tile, split);
+  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+    free_event(c);
+    return SHARPY_ECUDA;
   }
+  ev.tile_mixed = c->d_tile;
+  ev.tile_split = split;
   c->has_data = true;
   return SHARPY_OK;
 }

@@ -29,11 +29,8 @@ struct sharpy_ctx {
   // event tables (device)
   double* d_f = nullptr;
   double* d_b64 = nullptr;
-  float* d_b32 = nullptr;
-  float* d_b32lo = nullptr;
   double2* d_e64 = nullptr;
-  float2* d_e32 = nullptr;
-  unsigned char* d_stage = nullptr;  // staged records of a long segment
+  float4* d_tile = nullptr;  // the mixed sweep's tiles, then the split sweep's
   double* d_pref = nullptr;
   // status word and evidence accumulator (device)
   int* d_status = nullptr;

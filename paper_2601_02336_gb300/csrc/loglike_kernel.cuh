@@ -6,7 +6,6 @@
 #pragma once
 #include "bulk.cuh"
 #include "context.cuh"
-#include "split_stage.cuh"
 #include "sweep.cuh"
 
 namespace sharpy {
@@ -20,7 +19,7 @@ constexpr int kWarps = 8;
 // moments, hence ln L and the gradient, do not depend on SPLIT, which the
 // call's autotuner picks per (bins, detectors, particles, precision).
 template <int PREC, bool GRAD, int NDET, int SPLIT>
-__global__ void __launch_bounds__(kWarps * 32)
+__global__ void __launch_bounds__(kWarps * 32, PREC == SHARPY_FP64 ? 1 : 2)
 loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ theta, double* __restrict__ lnl,
                double* __restrict__ grad, int* status) {
   using DT = typename std::conditional<PREC == SHARPY_FP64, double, float>::type;
@@ -111,7 +110,7 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
 }
 
 // Staged variant for long segments on the mixed and split paths
-// (warps-per-vector choice kSplitStaged): one vector per warp, kWarps vectors per CTA walking
+// (warps-per-vector choice kSplitStaged): one vector per warp, kStagedWarps vectors per CTA walking
 // the same bins in step. Each block of kStageBins bins of the tables comes
 // into shared memory by one bulk copy (two buffers, each completed on an
 // mbarrier) and is read there by all the CTA's vectors, instead of by each
@@ -119,14 +118,14 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
 // s: chunks s, s + kStreams, ...; the 8 blocks of a chunk in order), each
 // vector runs mixed_bin on the same bins in the same order and flushes at the
 // same chunk ends, and the streams are added in order in FP64: the moments
-// equal those of the other choices bit for bit. The split path (SPLIT) reads
-// its own records (split_stage.cuh), which carry the lo parts of every basis
-// function instead of the FP64 tables.
+// equal those of the other choices bit for bit.
 constexpr int kSplitStaged = 16;
+constexpr int kStagedWarps = 8;
 
 // The walk over the blocks for a CTA whose vectors' last active bin is kmax.
 struct StageWalk {
   int kmax, st, c, b;
+  StageWalk() = default;
   __device__ explicit StageWalk(int km) : kmax(km), st(0), c(0), b(0) {}
   __device__ bool valid() const { return st < kStreams && c * kChunkBins + b * kStageBins <= kmax; }
   __device__ int block() const { return c * (kChunkBins / kStageBins) + b; }
@@ -140,25 +139,28 @@ struct StageWalk {
 };
 
 template <bool GRAD, int NDET, bool SPLIT>
-__global__ void __launch_bounds__(kWarps * 32, 2)
+__global__ void __launch_bounds__(kStagedWarps * 32, 2)
 loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ theta, double* __restrict__ lnl,
                       double* __restrict__ grad, int* status, int skip_block, int wait_polls) {
   constexpr int NACC = MomCount<NDET, GRAD>::value;
   using FS = FlushShape<NACC>;
   constexpr int NOUT = FS::KEEP;
-  constexpr int REC = SPLIT ? split_rec_bytes(NDET) : stage_rec_bytes(NDET);
-  using Ld = typename std::conditional<SPLIT, StagedSplitBin, StagedBin>::type;
-  const unsigned char* recs = ev.stage + (SPLIT ? split_set_offset(ev.stage_blocks, NDET) : 0);
+  constexpr int REC = stage_bytes(SPLIT);
+  const unsigned char* recs = reinterpret_cast<const unsigned char*>(SPLIT ? ev.tile_split : ev.tile_mixed);
   extern __shared__ __align__(128) unsigned char stage_buf[];  // two records
   __shared__ __align__(8) uint64_t full[2];
-  __shared__ SweepCoef sc[kWarps];
-  __shared__ EpiCoef<float> ec[kWarps];
-  __shared__ float mom[kWarps][NDET * kNMom * 2];
+  __shared__ SweepCoef sc[kStagedWarps];
+  __shared__ EpiCoef<float> ec[kStagedWarps];
+  __shared__ float mom[kStagedWarps][NDET * kNMom * 2];
+  __shared__ float outer_s[kStagedWarps][2 * NOUT][32];
+  __shared__ double tot_s[kStagedWarps][NOUT][32];
+  __shared__ StageWalk issue_s;
+  __shared__ int issued_s[2];  // phases armed per buffer
   __shared__ int kmax_s, abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t base = (int64_t)blockIdx.x * kWarps;
+  const int64_t base = (int64_t)blockIdx.x * kStagedWarps;
   const int D = m.n_dim;
-  if (warp == 0 && lane < kWarps) {
+  if (warp == 0 && lane < kStagedWarps) {
     const int64_t p = base + lane;
     if (p < n) {
       double th[kMaxDim];
@@ -178,7 +180,7 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
   }
   __syncthreads();
   if (warp == 0) {
-    int km = (lane < kWarps && sc[lane].ok) ? sc[lane].kisco : -1;
+    int km = (lane < kStagedWarps && sc[lane].ok) ? sc[lane].kisco : -1;
 #pragma unroll
     for (int o = 16; o >= 1; o >>= 1) km = max(km, __shfl_xor_sync(0xffffffffu, km, o));
     if (lane == 0) kmax_s = km;
@@ -187,63 +189,67 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
   const int kmax = kmax_s;
   const bool live = sc[warp].ok != 0;
   const int kend = live ? sc[warp].kisco : -1;
-  MixedCoef<NDET> P;
-  if (live) mixed_coef<NDET>(sc[warp], P);
+  const MixedCoef<NDET, SPLIT> P(sc[warp]);
   // the first two blocks; then block i + 2 into the buffer that block i leaves
-  StageWalk issue(kmax);
-  int issued[2] = {0, 0};  // phases armed per buffer (thread 0)
+  // (thread 0 walks the issues; its state stays in shared memory)
   // skip_block (failure-detection tests only): that block's copy is left out,
   // so the waits for it run out
-  if (threadIdx.x == 0)
-    for (int q = 0; q < 2 && issue.valid(); ++q, issue.next()) {
-      if (issue.block() == skip_block) continue;
+  auto issue_block = [&](int q) {
+    const int g = issue_s.block();
+    if (g != skip_block) {
       mbar_arrive_expect_tx(&full[q], REC);
-      bulk_copy_g2s(stage_buf + q * REC, recs + (size_t)issue.block() * REC, REC, &full[q]);
-      ++issued[q];
+      bulk_copy_g2s(stage_buf + q * REC, recs + (size_t)g * REC, REC, &full[q]);
+      ++issued_s[q];
     }
+    issue_s.next();
+  };
+  if (threadIdx.x == 0) {
+    issue_s = StageWalk(kmax);
+    issued_s[0] = issued_s[1] = 0;
+    for (int q = 0; q < 2 && issue_s.valid(); ++q) issue_block(q);
+  }
   bool timed_out = false;
-  float acc[NACC], hi[NOUT], lo[NOUT];
-  double tot[NOUT];
+  MomAcc<GRAD, NDET, SPLIT> acc;
+  acc.zero();
+  // outer sums of the chunk, the stream and the vector, touched once a chunk:
+  // in shared memory, so that the bins' sums and constants keep the registers
+  float(*hl)[32] = outer_s[warp];
+  double(*tot)[32] = tot_s[warp];
 #pragma unroll
-  for (int t = 0; t < NOUT; ++t) tot[t] = 0.0;
-  int i = 0;  // blocks consumed
-  for (int st = 0; st < kStreams && st * kChunkBins <= kmax; ++st) {
-#pragma unroll
-    for (int t = 0; t < NOUT; ++t) hi[t] = lo[t] = 0.0f;
-    for (int c = st; c * kChunkBins <= kmax; c += kStreams) {
-      const bool mine = c * kChunkBins <= kend;  // a chunk of this vector's sweep
-#pragma unroll
-      for (int a = 0; a < NACC; ++a) acc[a] = 0.0f;
-      for (int b = 0; b < kChunkBins / kStageBins && c * kChunkBins + b * kStageBins <= kmax; ++b, ++i) {
-        const int buf = i & 1;
-        if (!timed_out && !mbar_wait(&full[buf], (uint32_t)(i >> 1) & 1u, wait_polls)) {
-          timed_out = true;
-          abort_s = 1;
-        }
-        const unsigned char* rec = stage_buf + buf * REC;
-        if (mine && !timed_out) {
-          for (int u = 0; u < kStageBins / 32; ++u) {
-            const int k0 = c * kChunkBins + b * kStageBins + u * 32;
-            if (k0 > kend) break;
-            const int k = k0 + lane;
-            if (k <= kend) mixed_bin<GRAD, NDET, SPLIT>(sc[warp], P, Ld{rec, u * 32 + lane}, acc);
-          }
-        }
-        __syncthreads();  // every warp is done with this buffer
-        if (threadIdx.x == 0 && issue.valid() && !abort_s) {
-          if (issue.block() != skip_block) {
-            mbar_arrive_expect_tx(&full[buf], REC);
-            bulk_copy_g2s(stage_buf + buf * REC, recs + (size_t)issue.block() * REC, REC, &full[buf]);
-            ++issued[buf];
-          }
-          issue.next();
-        }
-      }
-      if (mine) flush<NACC>(acc, hi, lo, lane);
+  for (int t = 0; t < NOUT; ++t) hl[t][lane] = hl[NOUT + t][lane] = 0.0f, tot[t][lane] = 0.0;
+  StageWalk at(kmax);
+  for (int i = 0; at.valid(); ++i) {
+    const int buf = i & 1, g = at.block();
+    const int k0 = g * kStageBins + lane;
+    if (!timed_out && !mbar_wait(&full[buf], (uint32_t)(i >> 1) & 1u, wait_polls)) {
+      timed_out = true;
+      abort_s = 1;
     }
-    if (st * kChunkBins <= kend)
+    if (!timed_out) {
+      const float4* rec = reinterpret_cast<const float4*>(stage_buf + buf * REC) + lane;
+      const int kstop = min(kend, g * kStageBins + kStageBins - 1);
+#pragma unroll 1
+      for (int k = k0; k <= kstop; k += 32, rec += tile_quads(SPLIT) * kTileBins)
+        mixed_bin<GRAD, NDET, SPLIT>(P, StagedTile{rec}, acc);
+    }
+    __syncthreads();  // every warp is done with this buffer
+    if (threadIdx.x == 0 && issue_s.valid() && !abort_s) issue_block(buf);
+    const int c = g / (kChunkBins / kStageBins);
+    at.next();
+    // the last block of a chunk: its lane sums join the stream's; of a stream: the vector's
+    if ((!at.valid() || at.block() / (kChunkBins / kStageBins) != c) && c * kChunkBins <= kend) {
+      float hi[NOUT], lo[NOUT];
 #pragma unroll
-      for (int t = 0; t < NOUT; ++t) tot[t] += (double)hi[t] + (double)lo[t];
+      for (int t = 0; t < NOUT; ++t) hi[t] = hl[t][lane], lo[t] = hl[NOUT + t][lane];
+      flush_acc<SPLIT>(acc, hi, lo, lane);
+      const bool last = c + kStreams > kend / kChunkBins;  // the vector's last chunk of this stream
+#pragma unroll
+      for (int t = 0; t < NOUT; ++t) {
+        if (last) tot[t][lane] += (double)hi[t] + (double)lo[t];
+        hl[t][lane] = last ? 0.0f : hi[t];
+        hl[NOUT + t][lane] = last ? 0.0f : lo[t];
+      }
+    }
   }
   if (timed_out) set_status(status, SHARPY_ETIMEOUT);
   // after a timeout, wait (bounded, with the full bound whatever wait_polls
@@ -252,16 +258,16 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
   __syncthreads();
   if (threadIdx.x == 0 && abort_s)
     for (int q = 0; q < 2; ++q)
-      if (issued[q] > 0) mbar_wait(&full[q], (uint32_t)(issued[q] - 1) & 1u, kMbarWaitPolls);
+      if (issued_s[q] > 0) mbar_wait(&full[q], (uint32_t)(issued_s[q] - 1) & 1u, kMbarWaitPolls);
   if (live && FS::owner(lane)) {
 #pragma unroll
     for (int t = 0; t < NOUT; ++t) {
       const int idx = FS::index(lane, t);
-      if (idx < NACC) mom[warp][acc_to_mom<NDET, GRAD>(idx)] = (float)tot[t];
+      if (idx < NACC) mom[warp][acc_to_mom<NDET, GRAD>(idx)] = (float)tot[t][lane];
     }
   }
   __syncthreads();
-  if (warp == 0 && lane < kWarps) {
+  if (warp == 0 && lane < kStagedWarps) {
     const int64_t q = base + lane;
     if (q < n) {
       double l = NAN, gph[SHARPY_NPHYS];
@@ -283,11 +289,11 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
 template <bool GRAD, int NDET, bool SPLIT>
 inline cudaError_t launch_ll_staged(sharpy_ctx* c, int64_t n, const double* th, double* lnl, double* grad,
                                     cudaStream_t s) {
-  constexpr int bytes = 2 * (SPLIT ? split_rec_bytes(NDET) : stage_rec_bytes(NDET));
+  constexpr int bytes = 2 * stage_bytes(SPLIT);
   const cudaError_t e = cudaFuncSetAttribute(loglike_staged_kernel<GRAD, NDET, SPLIT>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  loglike_staged_kernel<GRAD, NDET, SPLIT><<<(unsigned)((n + kWarps - 1) / kWarps), kWarps * 32, bytes, s>>>(
+  loglike_staged_kernel<GRAD, NDET, SPLIT><<<(unsigned)((n + kStagedWarps - 1) / kStagedWarps), kStagedWarps * 32, bytes, s>>>(
       c->model, c->ev, n, th, lnl, grad, c->d_status, c->stage_skip_block,
       c->stage_wait_polls > 0 ? c->stage_wait_polls : kMbarWaitPolls);
   return cudaGetLastError();
@@ -311,10 +317,10 @@ inline cudaError_t launch_ll_split(sharpy_ctx* c, int split, int64_t n, const do
                                    cudaStream_t s) {
   if (split == kSplitStaged) {
     if constexpr (PREC == SHARPY_MIXED) {
-      if (c->ev.stage) return launch_ll_staged_unit(c, GRAD, NDET, n, th, lnl, grad, s);
+      if (c->ev.n_bins >= kStageMinBins) return launch_ll_staged_unit(c, GRAD, NDET, n, th, lnl, grad, s);
     }
     if constexpr (PREC == SHARPY_MIXED_SPLIT) {
-      if (c->ev.stage) return launch_ll_staged_split_unit(c, GRAD, NDET, n, th, lnl, grad, s);
+      if (c->ev.n_bins >= kStageMinBins) return launch_ll_staged_split_unit(c, GRAD, NDET, n, th, lnl, grad, s);
     }
     split = 8;  // no staged tables, or the FP64 path: the 8-warp split
   }

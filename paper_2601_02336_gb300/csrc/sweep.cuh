@@ -1,6 +1,7 @@
 // The per-bin sweep: one warp accumulates the moments of one particle.
 //
-// Lane l visits bins k = l, l+32, ... <= k_ISCO (coalesced SoA table reads).
+// Lane l visits bins k = l, l+32, ... <= k_ISCO (the mixed paths read tiles of
+// 32 bins, common.cuh; the FP64 path SoA tables).
 // Per bin the phase polynomial sum_j alpha_j B_j(f_k) + c0 is shared by all
 // detectors; per detector it adds f_k tau_a, reduces mod 1 turn, forms the
 // carrier e^{-i Psi}, multiplies the pre-whitened data E_ak and accumulates
@@ -127,197 +128,312 @@ __device__ __forceinline__ float frac_turn(float x) {
   return __fsub_rn(x, __fsub_rn(__fadd_rn(x, kRound32), kRound32));
 }
 
+// Two FP32 values in one 64-bit register pair. The packed instructions round
+// each half as the scalar ones do and issue once for both, at the same FP32
+// rate per lane: they pay where issue binds.
+using f32x2 = unsigned long long;
+__device__ __forceinline__ f32x2 pack2(float a, float b) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 dup2(float a) { return pack2(a, a); }
+__device__ __forceinline__ float2 unpack2(f32x2 v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// frac_turn of both halves (odd: frac2(-x) = -frac2(x))
+__device__ __forceinline__ f32x2 frac2(f32x2 x) {
+  const f32x2 r = add2(add2(x, dup2(kRound32)), dup2(-kRound32));
+  return fma2(r, dup2(-1.0f), x);
+}
+
+// A bin's quads: from the tiles in global memory, or from a block of tiles in
+// shared memory. Both sweeps walk tiles of 32 bins, lane = bin, so a quad is one
+// coalesced 16-byte load at a constant offset from the lane's pointer.
+struct GlobalTile {
+  const float4* at;  // quad 0 of the lane's bin
+  __device__ __forceinline__ float4 quad(int i) const { return __ldg(at + i * kTileBins); }
+  __device__ __forceinline__ ulonglong2 pair(int i) const {
+    return __ldg(reinterpret_cast<const ulonglong2*>(at + i * kTileBins));
+  }
+};
+struct StagedTile {
+  const float4* at;
+  __device__ __forceinline__ float4 quad(int i) const { return at[i * kTileBins]; }
+  __device__ __forceinline__ ulonglong2 pair(int i) const {
+    return *reinterpret_cast<const ulonglong2*>(at + i * kTileBins);
+  }
+};
+
+// Per-lane moment sums of NDET detectors. Mixed sweep with the gradient: pairs
+// in the tile's order, one packed FMA for two moments (per bin and detector 10
+// issues instead of 20; its FP64 terms leave the FP32 pipe slack that the
+// packed form's longer latency needs: 12.8 against 14.4 ms on 8192 vectors of
+// the 259585-bin segment). Otherwise single sums: the split sweep, whose FP32
+// pipe is the busier one, is faster with scalar FMAs (3.50 against 3.73 ms on
+// 1824 vectors).
+template <bool GRAD, int NDET, bool SPLIT>
+struct MomAcc {
+  float v[MomCount<NDET, GRAD>::value];
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int i = 0; i < MomCount<NDET, GRAD>::value; ++i) v[i] = 0.0f;
+  }
+  // adds the products of z = (zr, zi) with the bin's basis values b (tile pairs) and f, and z itself
+  __device__ __forceinline__ void add(int a, float zr, float zi, const f32x2* b, float f) {
+    if (GRAD) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 x = unpack2(b[i]);
+        const int j0 = mom_index(a, tile_basis(SPLIT, 2 * i), 0), j1 = mom_index(a, tile_basis(SPLIT, 2 * i + 1), 0);
+        v[j0] = fmaf(zr, x.x, v[j0]);
+        v[j0 + 1] = fmaf(zi, x.x, v[j0 + 1]);
+        v[j1] = fmaf(zr, x.y, v[j1]);
+        v[j1 + 1] = fmaf(zi, x.y, v[j1 + 1]);
+      }
+      const int jf = mom_index(a, 8, 0);
+      v[jf] = fmaf(zr, f, v[jf]);
+      v[jf + 1] = fmaf(zi, f, v[jf + 1]);
+      v[jf + 2] += zr;
+      v[jf + 3] += zi;
+    } else {
+      v[a * 2] += zr;
+      v[a * 2 + 1] += zi;
+    }
+  }
+  __device__ __forceinline__ void get(float* out) const {
+#pragma unroll
+    for (int i = 0; i < MomCount<NDET, GRAD>::value; ++i) out[i] = v[i];
+  }
+};
+template <int NDET>
+struct MomAcc<true, NDET, false> {
+  f32x2 m[NDET][2][kNMom / 2];  // pair 4: (f, 1)
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int a = 0; a < NDET; ++a)
+#pragma unroll
+      for (int i = 0; i < kNMom / 2; ++i) m[a][0][i] = m[a][1][i] = 0ULL;
+  }
+  __device__ __forceinline__ void add(int a, float zr, float zi, const f32x2* b, float f) {
+    const f32x2 z[2] = {dup2(zr), dup2(zi)};
+    const f32x2 f1 = pack2(f, 1.0f);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) m[a][r][i] = fma2(z[r], b[i], m[a][r][i]);
+      m[a][r][4] = fma2(z[r], f1, m[a][r][4]);  // the second half adds z itself
+    }
+  }
+  __device__ __forceinline__ void get(float* out) const {
+#pragma unroll
+    for (int a = 0; a < NDET; ++a)
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int i = 0; i < kNMom / 2; ++i) {
+          const float2 x = unpack2(m[a][r][i]);
+          out[mom_index(a, i < 4 ? tile_basis(false, 2 * i) : 8, r)] = x.x;
+          out[mom_index(a, i < 4 ? tile_basis(false, 2 * i + 1) : 9, r)] = x.y;
+        }
+  }
+};
+
+// Adds the lane sums to the outer accumulators and clears them.
+template <bool SPLIT, bool GRAD, int NDET>
+__device__ __forceinline__ void flush_acc(MomAcc<GRAD, NDET, SPLIT>& acc, float* hi, float* lo, int lane) {
+  constexpr int NACC = MomCount<NDET, GRAD>::value;
+  float v[NACC];
+  acc.get(v);
+  flush<NACC>(v, hi, lo, lane);
+  acc.zero();
+}
+
+// Per-particle constants of the sweep, in registers. The pairs follow the
+// tile's order; n*: negated (a product p = a b is formed as -p, so that its FMA
+// error term needs no negation).
+template <int NDET, bool SPLIT>
+struct MixedCoef {
+  static constexpr int NP = SPLIT ? 4 : 2;  // pairs of terms in FP32 pairs
+  f32x2 ah[NP], nah[NP], al[NP];
+  f32x2 th2, nth2, tl2;  // delays of detectors 0 and 1
+  float th, tl;          // delay of the odd detector
+  float c0f;             // split: c0 mod 1 turn
+  double alpha[4], s0;   // mixed: the large terms, c0 on the turn offset
+
+  __device__ __forceinline__ explicit MixedCoef(const SweepCoef& sc) {
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      const int j0 = tile_basis(SPLIT, 2 * i), j1 = tile_basis(SPLIT, 2 * i + 1);
+      ah[i] = pack2(sc.ahi[j0], sc.ahi[j1]);
+      nah[i] = pack2(-sc.ahi[j0], -sc.ahi[j1]);
+      al[i] = pack2(sc.alo[j0], sc.alo[j1]);
+    }
+    constexpr int d1 = NDET > 1 ? 1 : 0;
+    th2 = pack2(sc.thi[0], sc.thi[d1]);
+    nth2 = pack2(-sc.thi[0], -sc.thi[d1]);
+    tl2 = pack2(sc.tlo[0], sc.tlo[d1]);
+    th = sc.thi[NDET - 1];
+    tl = sc.tlo[NDET - 1];
+    if (SPLIT) {
+      c0f = sc.c0f;
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) alpha[i] = sc.alpha[large_pn(i)];
+      s0 = sc.c0 + kTurnOffset;
+    }
+  }
+};
+
+// One bin of the mixed (or split) sweep: its phase, carrier and moment
+// updates, with the bin's quads from the loader ld (global memory or a
+// shared-memory stage: the same values, so the same sums).
+template <bool GRAD, int NDET, bool SPLIT, class L>
+__device__ __forceinline__ void mixed_bin(const MixedCoef<NDET, SPLIT>& P, const L& ld,
+                                          MomAcc<GRAD, NDET, SPLIT>& acc) {
+  const float4 qf = ld.quad(tile_quad_f(SPLIT));  // f hi, f lo, E of detector 0
+  const float4 qe = NDET > 1 ? ld.quad(tile_quad_f(SPLIT) + 1) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const ulonglong2 h0 = ld.pair(0), h1 = GRAD || SPLIT ? ld.pair(1) : make_ulonglong2(0ULL, 0ULL);
+  const f32x2 b[4] = {h0.x, h0.y, h1.x, h1.y};
+  const float f = qf.x, fl = qf.y;
+  // the terms in FP32 pairs: p = ahi bhi is exact up to its FMA error term, its
+  // integer turns are removed exactly; nf: minus the fractions, er: the error
+  // and cross terms, of the pairs' halves
+  constexpr int NP = MixedCoef<NDET, SPLIT>::NP;
+  f32x2 nf[NP], er[NP];
+#pragma unroll
+  for (int i = 0; i < NP; i += 2) {
+    const ulonglong2 l = ld.pair(2 + i / 2);
+#pragma unroll
+    for (int u = i; u < i + 2; ++u) {
+      const f32x2 np = mul2(P.nah[u], b[u]);
+      nf[u] = frac2(np);
+      er[u] = fma2(P.ah[u], u == i ? l.x : l.y, fma2(P.al[u], b[u], fma2(P.ah[u], b[u], np)));
+    }
+  }
+  float ang[NDET];
+  const f32x2 ff = dup2(f), fll = dup2(fl), m1 = dup2(-1.0f);
+  if constexpr (!SPLIT) {
+    // the four terms that carry the large phase (Newtonian, 1PN, 1.5PN and
+    // the 2.5PN logarithm: up to ~2e3 turns on the long segment) accumulated
+    // in FP64 on the offset, whose low word is their fractional turn
+    const ulonglong2 q0 = ld.pair(5), q1 = ld.pair(6);
+    const unsigned long long q[4] = {q0.x, q0.y, q1.x, q1.y};
+    double S = P.s0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) S = fma(P.alpha[i], __longlong_as_double((long long)q[i]), S);
+    int turn_s = __double2loint(S);  // 2^-32 units
+    // the four terms below ~8 turns (2PN, 3PN, its logarithm, 3.5PN): the
+    // fractions summed pairwise in [-1/2, 1/2], then added to the FP64 part in
+    // 32-bit fixed point
+    const float2 n2 = unpack2(frac2(add2(nf[0], nf[1]))), e2 = unpack2(add2(er[0], er[1]));
+    const float n = frac_turn(__fadd_rn(n2.x, n2.y));
+    const float qs = frac_turn(__fsub_rn(__fadd_rn(e2.x, e2.y), n));
+    turn_s += __float2int_rn(qs * 4294967296.0f);  // wraps mod 1 turn
+    // f tau_a mod 1 from (thi + tlo)(fhi + flo): p = thi fhi is exact up to e
+    // (FMA), the other products are below 2^-20 turn
+    float qa[NDET];
+    if constexpr (NDET > 1) {
+      const f32x2 np = mul2(P.nth2, ff);
+      const f32x2 e = fma2(P.th2, fll, fma2(P.tl2, ff, fma2(P.th2, ff, np)));
+      const float2 x = unpack2(mul2(frac2(fma2(frac2(np), m1, e)), dup2(4294967296.0f)));
+      qa[0] = x.x;
+      qa[1] = x.y;
+    }
+    if constexpr (NDET != 2) {
+      const float p = __fmul_rn(P.th, f);
+      const float e = fmaf(P.th, fl, fmaf(P.tl, f, fmaf(P.th, f, -p)));
+      qa[NDET - 1] = frac_turn(__fadd_rn(frac_turn(p), e)) * 4294967296.0f;
+    }
+#pragma unroll
+    for (int a = 0; a < NDET; ++a) {
+      const int turn = turn_s + __float2int_rn(qa[a]);  // wraps mod 1 turn
+      ang[a] = (float)turn * 1.46291807926715968e-9f;    // 2 pi / 2^32
+    }
+  } else {
+    // sum_j alpha_j B_j mod 1: the fractions summed pairwise, reduced to
+    // [-1/2, 1/2] at every level (three levels instead of an eight-step
+    // chain), the error and cross terms likewise pairwise in Sm; the tile's
+    // pairs are (0, 2) + (1, 3) and (4, 6) + (5, 7)
+    static_assert(kNPn == 8, "the pairwise tree below is written for eight basis terms");
+    const float2 n03 = unpack2(frac2(add2(nf[0], nf[1]))), n47 = unpack2(frac2(add2(nf[2], nf[3])));
+    const float2 e03 = unpack2(add2(er[0], er[1])), e47 = unpack2(add2(er[2], er[3]));
+    const float n = __fadd_rn(frac_turn(__fadd_rn(n03.x, n03.y)), frac_turn(__fadd_rn(n47.x, n47.y)));
+    const float F = frac_turn(__fsub_rn(P.c0f, n));
+    const float Sm = __fadd_rn(__fadd_rn(e03.x, e03.y), __fadd_rn(e47.x, e47.y));
+    if constexpr (NDET > 1) {
+      const f32x2 np = mul2(P.nth2, ff);
+      const f32x2 Sa = fma2(P.th2, fll, fma2(P.tl2, ff, add2(dup2(Sm), fma2(P.th2, ff, np))));
+      const f32x2 Fa = frac2(fma2(frac2(np), m1, dup2(F)));
+      const float2 x = unpack2(mul2(add2(Fa, Sa), dup2(6.28318530717958648f)));
+      ang[0] = x.x;
+      ang[1] = x.y;
+    }
+    if constexpr (NDET != 2) {
+      const float p = __fmul_rn(P.th, f);
+      float Sa = __fadd_rn(Sm, fmaf(P.th, f, -p));
+      Sa = fmaf(P.th, fl, fmaf(P.tl, f, Sa));
+      const float Fa = frac_turn(__fadd_rn(F, frac_turn(p)));
+      ang[NDET - 1] = (Fa + Sa) * 6.28318530717958648f;
+    }
+  }
+#pragma unroll
+  for (int a = 0; a < NDET; ++a) {
+    float sn, cs;
+    __sincosf(ang[a], &sn, &cs);
+    const float2 E = a == 0 ? make_float2(qf.z, qf.w) : a == 1 ? make_float2(qe.x, qe.y) : make_float2(qe.z, qe.w);
+    // E e^{-i ang}, the contraction fixed
+    const float zr = __fmaf_rn(E.x, cs, __fmul_rn(E.y, sn));
+    const float zi = __fmaf_rn(E.y, cs, -__fmul_rn(E.x, sn));
+    acc.add(a, zr, zi, b, f);
+  }
+}
+
 // One stream of a mixed sweep: the chunks c = s, s + kStreams, ... of 2048
 // bins (64 lane iterations: one FP32 block each) below k_ISCO, accumulated
 // into this lane's compensated outer sums hi, lo (kept lane-distributed as
 // the flush leaves them). Returns whether the stream had any bin.
-// Table values of one bin for the mixed sweep, from the SoA tables in global
-// memory (bin k).
-struct GlobalBin {
-  const DevEvent& ev;
-  int64_t K;
-  int k;
-  __device__ __forceinline__ float b32(int j) const { return __ldg(ev.b32 + (int64_t)j * K + k); }
-  __device__ __forceinline__ float b32lo(int j) const { return __ldg(ev.b32lo + (int64_t)j * K + k); }
-  __device__ __forceinline__ double b64(int j) const { return __ldg(ev.b64 + (int64_t)j * K + k); }
-  __device__ __forceinline__ float2 e32(int a) const { return __ldg(ev.e32 + (int64_t)a * K + k); }
-};
-
-// The same values from a staged record in shared memory (bin i of its block;
-// the mixed sweep's tables only: the split sweep also reads the large terms'
-// lo parts).
-struct StagedBin {
-  const unsigned char* rec;
-  int i;
-  __device__ __forceinline__ float b32(int j) const { return reinterpret_cast<const float*>(rec)[j * kStageBins + i]; }
-  __device__ __forceinline__ float b32lo(int j) const {
-    return reinterpret_cast<const float*>(rec + stage_off_lo())[stage_lo_row(j) * kStageBins + i];
-  }
-  __device__ __forceinline__ double b64(int j) const {
-    return reinterpret_cast<const double*>(rec + stage_off_b64())[stage_b64_row(j) * kStageBins + i];
-  }
-  __device__ __forceinline__ float2 e32(int a) const {
-    return reinterpret_cast<const float2*>(rec + stage_off_e32())[a * kStageBins + i];
-  }
-};
-
-// Per-particle constants of the mixed sweep, held in registers.
-template <int NDET>
-struct MixedCoef {
-  double al[kNPn];
-  double s0;
-  float ah[kNPn], alo[kNPn], th[NDET], tl[NDET];
-};
-
-template <int NDET>
-__device__ __forceinline__ void mixed_coef(const SweepCoef& sc, MixedCoef<NDET>& P) {
-#pragma unroll
-  for (int j = 0; j < kNPn; ++j) P.al[j] = sc.alpha[j];
-  P.s0 = sc.c0 + kTurnOffset;
-#pragma unroll
-  for (int j = 0; j < kNPn; ++j) {
-    P.ah[j] = sc.ahi[j];
-    P.alo[j] = sc.alo[j];
-  }
-#pragma unroll
-  for (int a = 0; a < NDET; ++a) {
-    P.th[a] = sc.thi[a];
-    P.tl[a] = sc.tlo[a];
-  }
-}
-
-// One bin of the mixed (or split) sweep: its phase, carrier and moment
-// updates, with the bin's table values from the loader ld (global memory or a
-// shared-memory stage: the same values, so the same sums).
-template <bool GRAD, int NDET, bool SPLIT, class L>
-__device__ __forceinline__ void mixed_bin(const SweepCoef& sc, const MixedCoef<NDET>& P, const L& ld, float* acc) {
-  const double (&al)[kNPn] = P.al;
-  const double s0 = P.s0;
-  const float (&ah)[kNPn] = P.ah;
-  const float (&alo)[kNPn] = P.alo;
-  const float (&th)[NDET] = P.th;
-  const float (&tl)[NDET] = P.tl;
-  float bf[kNBasis];
-  if (GRAD || SPLIT) {
-#pragma unroll
-    for (int j = 0; j < kNBasis; ++j) bf[j] = ld.b32(j);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) bf[small_pn(i)] = ld.b32(small_pn(i));
-    bf[8] = ld.b32(8);
-  }
-  const float fl = ld.b32lo(8);
-  // phase: FP64 accumulation on the turn offset, or split single precision
-  double S = s0;
-  int turn_s = 0;
-  float F = 0.0f, Sm = 0.0f;
-  if (!SPLIT) {
-    // the four terms that carry the large phase (Newtonian, 1PN, 1.5PN and
-    // the 2.5PN logarithm: up to ~2e3 turns on the long segment) accumulated
-    // in FP64 on the offset
-#pragma unroll
-    for (int i = 0; i < 4; ++i) S = fma(al[large_pn(i)], ld.b64(large_pn(i)), S);
-    turn_s = __double2loint(S);  // fractional turn of the large terms, 2^-32 units
-    // the four terms below ~8 turns (2PN, 3PN, its logarithm, 3.5PN) in FP32
-    // pairs: each product's integer turns removed exactly (FMA error term
-    // kept), the fractions summed pairwise in [-1/2, 1/2], then added to the
-    // FP64 part in 32-bit fixed point
-    float fr[4], er[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int j = small_pn(i);
-      const float bl = ld.b32lo(j);
-      const float p = __fmul_rn(ah[j], bf[j]);
-      fr[i] = frac_turn(p);
-      er[i] = fmaf(ah[j], bl, fmaf(alo[j], bf[j], fmaf(ah[j], bf[j], -p)));
-    }
-    const float f = frac_turn(__fadd_rn(frac_turn(__fadd_rn(fr[0], fr[1])), frac_turn(__fadd_rn(fr[2], fr[3]))));
-    const float q = frac_turn(__fadd_rn(f, __fadd_rn(__fadd_rn(er[0], er[1]), __fadd_rn(er[2], er[3]))));
-    turn_s += __float2int_rn(q * 4294967296.0f);  // wraps mod 1 turn
-  } else {
-    // sum_j alpha_j B_j mod 1: p = ahi*bhi is exact up to e (FMA), its integer
-    // part is removed exactly; the fractions are summed pairwise, reduced to
-    // [-1/2, 1/2] at every level (three levels instead of an eight-step
-    // chain), the error and cross terms likewise pairwise in Sm.
-    static_assert(kNPn == 8, "the pairwise tree below is written for eight basis terms");
-    float fr[kNPn], er[kNPn];
-#pragma unroll
-    for (int j = 0; j < kNPn; ++j) {
-      const float bl = ld.b32lo(j);
-      const float p = __fmul_rn(ah[j], bf[j]);
-      fr[j] = frac_turn(p);
-      er[j] = fmaf(ah[j], bl, fmaf(alo[j], bf[j], fmaf(ah[j], bf[j], -p)));
-    }
-    const float f01 = frac_turn(__fadd_rn(fr[0], fr[1])), f23 = frac_turn(__fadd_rn(fr[2], fr[3]));
-    const float f45 = frac_turn(__fadd_rn(fr[4], fr[5])), f67 = frac_turn(__fadd_rn(fr[6], fr[7]));
-    const float f03 = frac_turn(__fadd_rn(f01, f23)), f47 = frac_turn(__fadd_rn(f45, f67));
-    F = frac_turn(__fadd_rn(__fadd_rn(f03, f47), sc.c0f));
-    Sm = __fadd_rn(__fadd_rn(__fadd_rn(er[0], er[1]), __fadd_rn(er[2], er[3])),
-                   __fadd_rn(__fadd_rn(er[4], er[5]), __fadd_rn(er[6], er[7])));
-  }
-#pragma unroll
-  for (int a = 0; a < NDET; ++a) {
-    float ang;
-    if (!SPLIT) {
-      // f tau_a mod 1 from (thi + tlo)(fhi + flo): p = thi fhi is exact up
-      // to e (FMA), the other products are below 2^-20 turn
-      const float p = __fmul_rn(th[a], bf[8]);
-      const float e = fmaf(th[a], fl, fmaf(tl[a], bf[8], fmaf(th[a], bf[8], -p)));
-      const float q = frac_turn(__fadd_rn(frac_turn(p), e));  // [-1/2, 1/2] turn
-      const int turn = turn_s + __float2int_rn(q * 4294967296.0f);  // wraps mod 1 turn
-      ang = (float)turn * 1.46291807926715968e-9f;  // 2 pi / 2^32
-    } else {
-      const float p = __fmul_rn(th[a], bf[8]);
-      float Sa = Sm + fmaf(th[a], bf[8], -p);
-      Sa = fmaf(th[a], fl, fmaf(tl[a], bf[8], Sa));
-      const float Fa = frac_turn(__fadd_rn(F, frac_turn(p)));
-      ang = (Fa + Sa) * 6.28318530717958648f;
-    }
-    float sn, cs;
-    __sincosf(ang, &sn, &cs);
-    const float2 E = ld.e32(a);
-    const float zr = E.x * cs + E.y * sn;
-    const float zi = E.y * cs - E.x * sn;
-    if (GRAD) {
-#pragma unroll
-      for (int j = 0; j < kNBasis; ++j) {
-        acc[(a * kNMom + j) * 2] += zr * bf[j];
-        acc[(a * kNMom + j) * 2 + 1] += zi * bf[j];
-      }
-      acc[(a * kNMom + 9) * 2] += zr;
-      acc[(a * kNMom + 9) * 2 + 1] += zi;
-    } else {
-      acc[a * 2] += zr;
-      acc[a * 2 + 1] += zi;
-    }
-  }
-}
-
 template <bool GRAD, int NDET, bool SPLIT>
 __device__ bool mixed_stream(const DevEvent& ev, const SweepCoef& sc, int s, float* hi, float* lo) {
   constexpr int NACC = MomCount<NDET, GRAD>::value;
   constexpr int NOUT = FlushShape<NACC>::KEEP;
+  constexpr int TQ = tile_quads(SPLIT) * kTileBins;  // float4 per tile
   const int lane = threadIdx.x & 31;
-  const int64_t K = ev.n_bins;
-  float acc[NACC];
-#pragma unroll
-  for (int i = 0; i < NACC; ++i) acc[i] = 0.0f;
+  MomAcc<GRAD, NDET, SPLIT> acc;
+  acc.zero();
 #pragma unroll
   for (int i = 0; i < NOUT; ++i) hi[i] = lo[i] = 0.0f;
-  MixedCoef<NDET> P;
-  mixed_coef<NDET>(sc, P);
+  const MixedCoef<NDET, SPLIT> P(sc);
+  const float4* tiles = (SPLIT ? ev.tile_split : ev.tile_mixed) + lane;
   const int kend = sc.kisco;
   bool any = false;
   // Warp-uniform trip counts: lanes past k_ISCO idle but still join the flushes.
   for (int c = s; c * kChunkBins <= kend; c += kStreams) {
     any = true;
-    for (int it = 0; it < kFlush; ++it) {
-      const int k0 = c * kChunkBins + it * 32;
-      if (k0 > kend) break;
-      const int k = k0 + lane;
-      if (k <= kend) mixed_bin<GRAD, NDET, SPLIT>(sc, P, GlobalBin{ev, K, k}, acc);
-    }
-    flush<NACC>(acc, hi, lo, lane);
+    const float4* at = tiles + (int64_t)c * kFlush * TQ;
+    const int its = min(kFlush, (kend - c * kChunkBins) / 32 + 1);
+    int k = c * kChunkBins + lane;
+#pragma unroll 1
+    for (int it = 0; it < its; ++it, k += 32, at += TQ)
+      if (k <= kend) mixed_bin<GRAD, NDET, SPLIT>(P, GlobalTile{at}, acc);
+    flush_acc<SPLIT>(acc, hi, lo, lane);
   }
   return any;
 }

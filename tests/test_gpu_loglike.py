@@ -315,3 +315,30 @@ def test_staged_kernel_wait_timeout_reports_status():
     assert ctx.status() == 0
     assert torch.equal(l, ref_l) and torch.equal(g, ref_g)
     ctx.set_loglike_split(0)
+
+
+@pytest.mark.parametrize("n_bins", [1, 31, 32, 33, 255, 256, 257, 2047, 2048, 2049])
+@pytest.mark.parametrize("name", ["tiny", "bbh11"])
+def test_loglike_tile_edges(name, n_bins):
+    """The mixed and split sweeps read tiles of 32 bins in blocks of 256, flushed every 2048: segments around each
+    edge agree with the oracle on ln L (1e-3, the workloads' bound) and on the gradient (1e-4 of its norm in prior
+    widths, or 1e-3 where the norm is below the ln L bound's scale), one and three detectors, with and without the
+    gradient, on one warp and on eight warps a vector."""
+    G.require_gpu()
+    w = inputs.WORKLOADS[name]()
+    w.n_bins = n_bins
+    ev, ctx, th_inj, _ = G.event_pair(w, seed=0)
+    th = np.vstack([inputs.prior_draws(w, 6, 51), inputs.ball(w, th_inj, 5, 52)])
+    ref_l, ref_g = oracle.loglike(helpers.oracle_model(w), ev, th)
+    wid = G.width(w)
+    norm = np.linalg.norm(ref_g * wid, axis=1)
+    for prec in ("mixed", "split"):
+        for split in (1, 8):
+            ctx.set_loglike_split(split)
+            l, g = ctx.loglike_grad(G.to_dev(th), prec)
+            l0, _ = ctx.loglike_grad(G.to_dev(th), prec, grad=False)
+            assert np.max(np.abs(l.cpu().numpy() - ref_l)) <= 1e-3
+            assert np.max(np.abs(l0.cpu().numpy() - ref_l)) <= 1e-3
+            err = np.linalg.norm((g.cpu().numpy() - ref_g) * wid, axis=1)
+            assert np.all(err <= np.maximum(1e-4 * norm, 1e-3)), (prec, split)
+    assert ctx.status() == 0
