@@ -1,5 +1,5 @@
 // The standalone likelihood kernel (sharpy_loglike_grad): one CTA of kWarps
-// warps; warp 0 computes the per-particle prologue lane-parallel (lane s =
+// warps; warps 0 to 4 compute the particles' prologues (prologue_cta: lane s =
 // particle s of the CTA), the warps sweep the particles' bins, and warp 0
 // finishes with the lane-parallel epilogue. The instantiations of each
 // precision are compiled in their own unit (loglike_inst.cu).
@@ -35,17 +35,14 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = (int64_t)blockIdx.x * PPC;
   const int D = m.n_dim;
-  if (warp == 0 && lane < PPC) {
-    int64_t p = base + lane;
-    if (p < n) {
-      double th[kMaxDim];
-      for (int i = 0; i < D; ++i) th[i] = theta[p * D + i];
-      prologue<DT, GRAD, PREC == SHARPY_MIXED_SPLIT>(m, ev, th, sc[lane], ec[lane]);
-    } else {
-      sc[lane].ok = 0;
-      sc[lane].kisco = -1;
-    }
-  }
+  prologue_cta<DT, GRAD, PREC == SHARPY_MIXED_SPLIT>(
+      warp, lane, PPC, m, ev,
+      [&](int s, double* th) {
+        if (base + s >= n) return false;
+        for (int i = 0; i < D; ++i) th[i] = theta[(base + s) * D + i];
+        return true;
+      },
+      sc, ec);
   __syncthreads();
   const int pl = warp / SPLIT, r = warp % SPLIT;
   const int64_t p = base + pl;
@@ -160,17 +157,14 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t base = (int64_t)blockIdx.x * kStagedWarps;
   const int D = m.n_dim;
-  if (warp == 0 && lane < kStagedWarps) {
-    const int64_t p = base + lane;
-    if (p < n) {
-      double th[kMaxDim];
-      for (int i = 0; i < D; ++i) th[i] = theta[p * D + i];
-      prologue<float, GRAD, SPLIT>(m, ev, th, sc[lane], ec[lane]);
-    } else {
-      sc[lane].ok = 0;
-      sc[lane].kisco = -1;
-    }
-  }
+  prologue_cta<float, GRAD, SPLIT>(
+      warp, lane, kStagedWarps, m, ev,
+      [&](int s, double* th) {
+        if (base + s >= n) return false;
+        for (int i = 0; i < D; ++i) th[i] = theta[(base + s) * D + i];
+        return true;
+      },
+      sc, ec);
   for (int i = lane; i < NDET * kNMom * 2; i += 32) mom[warp][i] = 0.0f;
   if (threadIdx.x == 0) {
     mbar_init(&full[0], 1);

@@ -261,9 +261,14 @@ __global__ void __launch_bounds__(kMetWarps * 32)
   for (int i = 0; i < D; ++i) x[i] = theta[p * D + i];
   if (threadIdx.x == 0) S.ok[0] = S.ok[1] = 0xffffffffu;
   if (m.model == SHARPY_MODEL_TAYLORF2) {
-    // prologue: the phase half on warp 0, the sky half on warp 1
-    if (warp == 0) prologue_phase<double, true>(m, ev, x, S.pro.sc[lane], S.pro.ec[lane]);
-    if (warp == 1) prologue_sky<double, true>(m, ev, x, S.pro.sc[lane], S.pro.ec[lane]);
+    // prologue: the phase on warp 0, the amplitude and the detectors' sky on the others
+    if (warp == 0) {
+      prologue_phase<double, true>(m, ev, x, S.pro.sc[lane], S.pro.ec[lane]);
+    } else {
+      if (warp == 1) prologue_amp<double, true>(m, x, S.pro.ec[lane]);
+      prologue_sky<double, true>(m, ev, x, min(warp - 1, ev.n_det), min(warp, ev.n_det), S.pro.sc[lane],
+                                 S.pro.ec[lane]);
+    }
     __syncthreads();
     // Fisher matrices of the detectors on warps 0.., added in detector order
     double v[kTri];

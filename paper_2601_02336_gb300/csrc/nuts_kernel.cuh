@@ -829,10 +829,12 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
     if (gw && (warp == cw || warp == (cw ^ 1)) && lane < SLOTS && S.pending[lane]) {
       double x[kMaxDim];
       for (int i = 0; i < D; ++i) x[i] = S.pos[P_N][lane][i];
-      if (warp == cw)
+      if (warp == cw) {
         prologue_phase<DT, true, PREC == SHARPY_MIXED_SPLIT>(A.m, A.ev, x, sc[lane], ec[lane]);
-      else
-        prologue_sky<DT, true, PREC == SHARPY_MIXED_SPLIT>(A.m, A.ev, x, sc[lane], ec[lane]);
+      } else {
+        prologue_amp<DT, true>(A.m, x, ec[lane]);
+        prologue_sky<DT, true, PREC == SHARPY_MIXED_SPLIT>(A.m, A.ev, x, 0, A.ev.n_det, sc[lane], ec[lane]);
+      }
     }
     if (gw && warp == cw) {
       // order this tick's sweeps by decreasing k_ISCO (ties: slot order)
