@@ -36,8 +36,7 @@ int launch_nuts(int precision, int ndet, int slots, const NutsArgs& A, unsigned 
 constexpr int64_t kLongSignalBins = 65536;
 
 // slots: particles per CTA; 0 picks the autotuned count for (n, precision) if
-// the context has one, else the widest count that still gives about two CTAs
-// per SM.
+// the context has one, else by n (below).
 int enqueue_nuts(sharpy_ctx* c, int64_t n, const double* beta_ptr, double beta, double* theta, double* lnl,
                  double* grad, const double* inv_mass, const double* cov_step, double step, int max_depth,
                  int n_steps, uint64_t key, uint32_t ctr, int precision, sharpy_nuts_stats* stats, cudaStream_t s,
@@ -70,7 +69,15 @@ int enqueue_nuts(sharpy_ctx* c, int64_t n, const double* beta_ptr, double beta, 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    slots = n >= (int64_t)16 * 2 * sms * 3 / 4 ? 16 : 8;
+    // FP64: 16 slots once they give about 1.5 CTAs an SM. Mixed paths: 8 slots
+    // while one CTA an SM holds them (2048 particles: 3.03 ms with 8, 2.86 with
+    // 16; 700: 2.29 and 2.78), 16 while they fit one wave (three CTAs of four
+    // warps an SM; 5000: 5.19 ms, 5.88 with 32), then 32 (16384: 11.6 ms, 14.2
+    // with 16).
+    if (precision == SHARPY_FP64)
+      slots = n >= (int64_t)16 * 2 * sms * 3 / 4 ? 16 : 8;
+    else
+      slots = n <= (int64_t)8 * sms ? 8 : n <= (int64_t)16 * 3 * sms ? 16 : 32;
   }
   const int nd = c->model.model == SHARPY_MODEL_TAYLORF2 ? c->ev.n_det : 1;
   if (c->model.model == SHARPY_MODEL_TAYLORF2 && c->ev.n_bins >= kLongSignalBins) {

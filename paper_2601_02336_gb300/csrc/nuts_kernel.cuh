@@ -2,19 +2,20 @@
 // variant with biased progressive sampling at the top level and the
 // generalised U-turn criterion on every completed sub-tree).
 //
-// One CTA of kNutsWarps warps owns SLOTS (8, 16 or 32) particles for the
-// whole call; the slot count is autotuned (about two CTAs share each SM, so
-// their serial per-particle phases overlap with each other's sweeps). Every
+// One CTA of W warps owns SLOTS (4, 8, 16 or 32) particles for the whole call
+// (the geometries are in launch_nuts_impl); the slot count is autotuned (about
+// two CTAs share each SM, so their serial per-particle phases overlap with each
+// other's sweeps). Every
 // slot's trajectory is grown one leapfrog at a time (iteratively, no
 // recursion), and every leapfrog needs one likelihood+gradient evaluation.
 // Each "tick" of the CTA has three phases between barriers:
-//   A  the prologue of every pending evaluation, lane = slot: the phase half
-//      (PN coefficients, k_ISCO; FP64, or double-float on the mixed paths) on
-//      the control warp, the sky half (responses, delays, amplitude) on its
+//   A  the prologue of every pending evaluation, lane = slot: the phase (PN
+//      coefficients, k_ISCO; FP64, or double-float on the mixed paths) on the
+//      control warp, the amplitude and the sky (responses, delays) on its
 //      neighbour, a warp on another SM sub-partition;
 //   B  each warp sweeps the bins of the next pending particle, longest first;
 //   C  each pending slot's epilogue, tree update and first half of the next
-//      leapfrog, on a lane group of 32/(SLOTS/4) lanes (one or more dimensions
+//      leapfrog, on a lane group of 32/(SLOTS/W) lanes (one or more dimensions
 //      per lane), the pending slots dealt out one per warp first.
 // An FP64 warp instruction costs the same pipe time whatever its active-lane
 // count, and a warp runs the union of its lanes' branches of the state
@@ -45,7 +46,6 @@
 
 namespace sharpy {
 
-constexpr int kNutsWarps = 4;  // warps per CTA; two CTAs share an SM so their serial phases interleave
 constexpr int kMaxDepth = SHARPY_MAX_DEPTH;
 constexpr double kDivergence = 1000.0;
 
@@ -198,10 +198,10 @@ __device__ __forceinline__ void draw2(uint64_t key, uint32_t c0, uint32_t c1, ui
 constexpr int kLaneDims = 16;
 static_assert(kMaxDim <= kLaneDims, "one fixed reduction tree over at most 16 dimensions");
 
-template <int PREC, int NDET, int SLOTS>
+template <int PREC, int NDET, int SLOTS, int W>
 struct Nuts {
   using VT = typename std::conditional<PREC == SHARPY_FP64, double, float>::type;
-  static constexpr int SPW = SLOTS / kNutsWarps;  // slots per warp
+  static constexpr int SPW = SLOTS / W;  // slots per warp
   // lanes per slot: 16, 8, 4 (16 also for one slot per warp, whose group
   // leaves the upper half-warp out: the group size fixes the arithmetic)
   static constexpr int G = SPW == 1 ? 16 : 32 / SPW;
@@ -659,11 +659,15 @@ struct NutsSmem {
   MT mom[SLOTS][NDET * kNMom * 2];
 };
 
-// Mixed paths: registers for three CTAs per SM (168 a thread, no spills),
-// which the 8- and 16-slot launches can use (9 % on 16384 particles); FP64:
-// two.
-template <int PREC, int NDET, int SLOTS>
-__global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SLOTS == 4 ? 4 : 3))
+// CTAs per SM the registers are held to: 16 warps an SM at 128 registers (a
+// few words spilled in the state machine) for the eight-warp and the four-slot
+// launches; three CTAs of four warps (168, no spills); FP64: two.
+template <int PREC, int SLOTS, int W>
+__host__ __device__ constexpr int nuts_ctas() {
+  return PREC == SHARPY_FP64 || W == 8 ? 2 : SLOTS == 4 ? 4 : 3;
+}
+template <int PREC, int NDET, int SLOTS, int W>
+__global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
     nuts_kernel(const __grid_constant__ NutsArgs P) {
   using DT = typename std::conditional<PREC == SHARPY_FP64, double, float>::type;
   using VT = DT;
@@ -700,65 +704,95 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
   const int D = A.m.n_dim;
   const bool gw = A.m.model == SHARPY_MODEL_TAYLORF2;
 
-  // metric, its Cholesky factor (diagonal fallback; computed in FP64), step size, beta
-  if (threadIdx.x == 0) {
-    S.mstride = A.local_metric ? SLOTS : 1;
-    S.mmin = reinterpret_cast<VT*>(smem_raw + nuts_metric_offset<PREC, NDET, SLOTS>());
-    S.mchol = S.mmin + kMaxDim * kMaxDim * S.mstride;
-    double mi[kMaxDim][kMaxDim], ch[kMaxDim][kMaxDim];
-    for (int i = 0; i < D; ++i)
-      for (int j = 0; j < D; ++j) mi[i][j] = A.minv ? A.minv[i * D + j] : (i == j ? 1.0 : 0.0);
-    bool ok = true;
-    for (int j = 0; j < D && ok; ++j) {
-      for (int i = 0; i < D; ++i) ch[i][j] = 0.0;
-      double d = mi[j][j];
-      for (int k = 0; k < j; ++k) d -= ch[j][k] * ch[j][k];
-      if (!(d > 0.0) || !isfinite(d)) {
-        ok = false;
-        break;
+  // metric, its Cholesky factor (diagonal fallback; computed in FP64), step
+  // size, beta. Lane i of the control warp holds row i; a launch waits for this,
+  // so what it does not need is left out: no factorisation without a metric
+  // (the identity is its own factor) or with one per particle (loaded below).
+  if (warp == cw) {
+    const int mstride = A.local_metric ? SLOTS : 1;
+    VT* mmin = reinterpret_cast<VT*>(smem_raw + nuts_metric_offset<PREC, NDET, SLOTS>());
+    VT* mchol = mmin + kMaxDim * kMaxDim * mstride;
+    const int row = lane < D ? lane : D - 1;
+    int kind = METRIC_IDENTITY;
+    if (A.pminv) {
+      kind = METRIC_DENSE;
+    } else {
+      double mi[kMaxDim], ch[kMaxDim];  // row `row` (registers: constant indices only)
+#pragma unroll
+      for (int j = 0; j < kMaxDim; ++j) {
+        mi[j] = row == j ? 1.0 : 0.0;
+        if (A.minv && j < D) mi[j] = A.minv[row * D + j];
+        ch[j] = row == j ? 1.0 : 0.0;
       }
-      ch[j][j] = sqrt(d);
-      for (int i = j + 1; i < D; ++i) {
-        double t = mi[i][j];
-        for (int k = 0; k < j; ++k) t -= ch[i][k] * ch[j][k];
-        ch[i][j] = t / ch[j][j];
-      }
-    }
-    if (!ok)
-      for (int i = 0; i < D; ++i)
-        for (int j = 0; j < D; ++j) {
-          double dii = mi[i][i] > 0.0 && isfinite(mi[i][i]) ? mi[i][i] : 1.0;
-          mi[i][j] = i == j ? dii : 0.0;
-          ch[i][j] = i == j ? sqrt(dii) : 0.0;
+      if (A.minv) {
+        bool ok = true;
+#pragma unroll
+        for (int j = 0; j < kMaxDim; ++j) {
+          if (j >= D || !ok) break;
+          // column j: every row's t = mi[i][j] - sum_k ch[i][k] ch[j][k], the pivot's first
+          double t = mi[j];
+#pragma unroll
+          for (int k = 0; k < j; ++k) t -= ch[k] * __shfl_sync(0xffffffffu, ch[k], j);
+          const double d = __shfl_sync(0xffffffffu, t, j);
+          if (!(d > 0.0) || !isfinite(d)) {
+            ok = false;
+            break;
+          }
+          const double c = sqrt(d);
+          ch[j] = row == j ? c : row > j ? t / c : 0.0;
         }
-    bool ident = true, diag = true;
-    for (int i = 0; i < D; ++i)
-      for (int j = 0; j < D; ++j) {
-        if (i != j && mi[i][j] != 0.0) diag = false;
-        if (mi[i][j] != (i == j ? 1.0 : 0.0)) ident = false;
-        S.mmin[i * kMaxDim + j] = (VT)mi[i][j];  // the one copy (or slot 0's)
-        S.mchol[i * kMaxDim + j] = (VT)ch[i][j];
+        if (!ok) {
+          double dii = 1.0;
+#pragma unroll
+          for (int j = 0; j < kMaxDim; ++j)
+            if (row == j) dii = mi[j] > 0.0 && isfinite(mi[j]) ? mi[j] : 1.0;
+          const double r = sqrt(dii);
+#pragma unroll
+          for (int j = 0; j < kMaxDim; ++j) {
+            mi[j] = row == j ? dii : 0.0;
+            ch[j] = row == j ? r : 0.0;
+          }
+        }
       }
-    S.metric_kind = A.pminv ? METRIC_DENSE : ident ? METRIC_IDENTITY : (diag ? METRIC_DIAGONAL : METRIC_DENSE);
+      bool ident = true, diag = true;
+#pragma unroll
+      for (int j = 0; j < kMaxDim; ++j) {
+        if (j >= D) break;
+        if (row != j && mi[j] != 0.0) diag = false;
+        if (mi[j] != (row == j ? 1.0 : 0.0)) ident = false;
+        if (lane < D) {
+          mmin[row * kMaxDim + j] = (VT)mi[j];
+          mchol[row * kMaxDim + j] = (VT)ch[j];
+        }
+      }
+      ident = __all_sync(0xffffffffu, ident);
+      diag = __all_sync(0xffffffffu, diag);
+      kind = ident ? METRIC_IDENTITY : (diag ? METRIC_DIAGONAL : METRIC_DENSE);
+    }
+    // the prior's constant terms (summed in dimension order) and the step
+    const double lo = A.m.lo[row], hi = A.m.hi[row];
+    const double lt = A.m.prior[row] == SHARPY_PRIOR_POWER2 ? log(3.0 / (hi * hi * hi - lo * lo * lo)) : -log(hi - lo);
+    const double sd = A.cov_step ? sqrt(A.cov_step[row * D + row]) : 0.0;
+    if (lane < D) {
+      S.lokey[lane] = okey(lo);
+      S.hikey[lane] = okey(hi);
+    }
+    double lpc = 0.0, smin = INFINITY;
     for (int i = 0; i < D; ++i) {
-      S.lokey[i] = okey(A.m.lo[i]);
-      S.hikey[i] = okey(A.m.hi[i]);
+      lpc += __shfl_sync(0xffffffffu, lt, i);
+      smin = fmin(smin, __shfl_sync(0xffffffffu, sd, i));
     }
-    double lpc = 0.0;
-    for (int i = 0; i < D; ++i) {
-      double lo = A.m.lo[i], hi = A.m.hi[i];
-      lpc += A.m.prior[i] == SHARPY_PRIOR_POWER2 ? log(3.0 / (hi * hi * hi - lo * lo * lo)) : -log(hi - lo);
+    if (lane == 0) {
+      const double eps = A.cov_step ? A.step * smin : A.step;
+      S.mmin = mmin;
+      S.mchol = mchol;
+      S.mstride = mstride;
+      S.metric_kind = kind;
+      S.lp_const = lpc;
+      S.eps = eps;
+      S.epsv = (VT)eps;
+      S.beta = A.beta_ptr ? *A.beta_ptr : A.beta;
     }
-    S.lp_const = lpc;
-    double eps = A.step;
-    if (A.cov_step) {
-      double smin = INFINITY;
-      for (int j = 0; j < D; ++j) smin = fmin(smin, sqrt(A.cov_step[j * D + j]));
-      eps = A.step * smin;
-    }
-    S.eps = eps;
-    S.epsv = (VT)eps;
-    S.beta = A.beta_ptr ? *A.beta_ptr : A.beta;
   }
   __syncthreads();
 
@@ -766,9 +800,9 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
   // w SPW + SPW - 1, each on a group of G = 32 / SPW lanes that share its
   // vectors' dimensions, so the per-slot phases of a tick (epilogue, tree
   // update, next leapfrog) run on all four SM sub-partitions at once.
-  using NT = Nuts<PREC, NDET, SLOTS>;
+  using NT = Nuts<PREC, NDET, SLOTS, W>;
   constexpr int SPW = NT::SPW, G = NT::G, DPL = NT::DPL;
-  static_assert(SLOTS % kNutsWarps == 0, "slots are shared evenly by the warps");
+  static_assert(SLOTS % W == 0, "slots are shared evenly by the warps");
   const bool in_group = lane / G < SPW;   // false: the idle half-warp of a one-slot warp
   const int my = in_group ? warp * SPW + lane / G : -1;  // this lane's slot
   const int tg = lane % G;                // its lane within the slot's group
@@ -824,8 +858,8 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
     }
     __syncthreads();
     if (!S.alive) break;
-    // (A) prologues (GW models; lane = slot): the phase half on the control
-    // warp, the sky half on its neighbour, on another sub-partition
+    // (A) prologues (GW models; lane = slot): the phase on the control warp, the
+    // amplitude and the sky on its neighbour, on another sub-partition
     if (gw && (warp == cw || warp == (cw ^ 1)) && lane < SLOTS && S.pending[lane]) {
       double x[kMaxDim];
       for (int i = 0; i < D; ++i) x[i] = S.pos[P_N][lane][i];
@@ -877,7 +911,7 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
       __syncwarp();
       if (pd) {
         const int r = __popc(pm & ((1u << lane) - 1u));
-        S.cslot[(r % kNutsWarps) * SPW + r / kNutsWarps] = lane;
+        S.cslot[(r % W) * SPW + r / W] = lane;
       }
     }
     __syncthreads();
@@ -1011,20 +1045,41 @@ __global__ void __launch_bounds__(kNutsWarps * 32, PREC == SHARPY_FP64 ? 2 : (SL
 // combination.
 int launch_nuts(int precision, int ndet, int slots, const NutsArgs& A, unsigned grid, cudaStream_t s);
 
+// Launch geometry of a slot count. On the mixed paths 8, 16 and 32 slots run on
+// eight warps: a tick then has as many sweeps and state machines in flight again
+// as on four, for the same prologue (one lane a slot on one warp, bound by FP64
+// issue whatever its lane count). Two such CTAs fit an SM. 16 slots between two
+// and three CTAs an SM keep four warps, three of which fit: one wave instead of
+// two. Measured, ms, four / eight warps: 2048 particles, 16 slots 4.11 / 2.86
+// (8 slots on four warps 2.97); 16384 particles at 16 s, 16 slots 72.3 / 63.6,
+// 32 slots 82.3 / 62.4; 700 particles, 8 slots 2.45 / 2.29; 5000 particles (313
+// CTAs), 16 slots 5.19 / 6.11. FP64 (its sums need 255 registers) and 4 slots:
+// four warps.
 template <int P, int ND>
 int launch_nuts_impl(int slots, const NutsArgs& A, unsigned grid, cudaStream_t s) {
-  auto go = [&](auto kernel, int sl, size_t bytes) -> int {
+  auto go = [&](auto kernel, int sl, int warps, size_t bytes) -> int {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
       return SHARPY_ECUDA;
     const unsigned g = grid ? grid : (unsigned)((A.n + sl - 1) / sl);
-    kernel<<<g, kNutsWarps * 32, bytes, s>>>(A);
+    kernel<<<g, warps * 32, bytes, s>>>(A);
     return cudaGetLastError() == cudaSuccess ? SHARPY_OK : SHARPY_ECUDA;
   };
   const bool local = A.local_metric != 0;
-  if (slots == 4) return go(nuts_kernel<P, ND, 4>, 4, nuts_smem_bytes<P, ND, 4>(local));
-  if (slots == 32) return go(nuts_kernel<P, ND, 32>, 32, nuts_smem_bytes<P, ND, 32>(local));
-  if (slots == 16) return go(nuts_kernel<P, ND, 16>, 16, nuts_smem_bytes<P, ND, 16>(local));
-  return go(nuts_kernel<P, ND, 8>, 8, nuts_smem_bytes<P, ND, 8>(local));
+  constexpr int W = P == SHARPY_FP64 ? 4 : 8;
+  if (slots == 4) return go(nuts_kernel<P, ND, 4, 4>, 4, 4, nuts_smem_bytes<P, ND, 4>(local));
+  if (slots == 32) return go(nuts_kernel<P, ND, 32, W>, 32, W, nuts_smem_bytes<P, ND, 32>(local));
+  if (slots == 16) {
+    if constexpr (W == 8) {
+      int dev = 0, sms = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return SHARPY_ECUDA;
+      const int64_t g = grid ? grid : (A.n + 15) / 16;
+      if (g > 2 * sms && g <= 3 * sms) return go(nuts_kernel<P, ND, 16, 4>, 16, 4, nuts_smem_bytes<P, ND, 16>(local));
+    }
+    return go(nuts_kernel<P, ND, 16, W>, 16, W, nuts_smem_bytes<P, ND, 16>(local));
+  }
+  return go(nuts_kernel<P, ND, 8, W>, 8, W, nuts_smem_bytes<P, ND, 8>(local));
 }
 
 }  // namespace sharpy

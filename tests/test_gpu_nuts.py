@@ -364,3 +364,25 @@ def test_nuts_slot_count_invariant():
             assert np.array_equal(st[f], ref[3][f]), (slots, f)
     ctx.set_nuts_slots(0)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("n", [1, 9, 33, 16 * 2 * 152 + 1, 16 * 3 * 152, 16 * 3 * 152 + 1])
+def test_nuts_geometry_invariant(n):
+    """The launch's geometry (8, 16 or 32 slots on eight warps, 16 on four between two and three CTAs per SM of a
+    152-SM GPU, 4 on four) and the count that the call picks by itself give the same particles and statistics, bit
+    for bit, at counts around its edges and with a ragged last CTA."""
+    G.require_gpu()
+    w = inputs.tiny()
+    ctx, th_inj, _ = api.make_event(w, seed=0)
+    t0 = G.to_dev(inputs.prior_draws(w, n, 61))
+    for prec in ("mixed", "split"):
+        l0, g0 = ctx.loglike_grad(t0, prec)
+        ref = None
+        for slots in (0, 4, 8, 16, 32):
+            ctx.set_nuts_slots(slots)
+            t, l, g = t0.clone(), l0.clone(), g0.clone()
+            st = ctx.nuts_mutate(0.3, t, l, g, None, 1e-3, 3, 2, key=5, ctr=9, precision=prec)
+            got = (t, l, g, st)
+            ref = ref or got
+            assert all(torch.equal(a, b) for a, b in zip(got, ref)), (prec, slots)
+    assert ctx.status() == 0
