@@ -22,6 +22,7 @@ constexpr int kMaxDim = SHARPY_MAX_DIM;
 constexpr int kMaxDet = SHARPY_MAX_DET;
 constexpr int kNBasis = 9;  // x^5, x^3, x^2, x, ln f, y, y ln f, y^2, f  (x = f^-1/3, y = f^1/3)
 constexpr int kNPn = 8;     // the first eight: post-Newtonian phase basis
+constexpr int kNMom = kNBasis + 1;  // moments per detector: Y_aj of the basis, then Z_a
 // The mixed sweep's split of the post-Newtonian basis: terms accumulated in
 // FP64 (x^5, x^3, x^2, ln f) and terms formed in FP32 pairs (x, y, y ln f, y^2).
 __host__ __device__ constexpr int large_pn(int i) { return i < 3 ? i : 4; }
@@ -76,6 +77,8 @@ struct DevDetector {
   float rcf[3];    // the same in FP32 (delays of the mixed path)
 };
 
+struct FixBlock;  // fixed.cuh
+
 // Staged event tables (device pointers, SoA), built by sharpy_set_data.
 struct DevEvent {
   int n_det;
@@ -89,6 +92,9 @@ struct DevEvent {
   const double2* e64;        // [n_det][K] E = w conj(d) f^-7/6 (FP64)
   const float4* tile_mixed;  // tiles of the mixed and the split sweep, whole blocks of kStageBins
   const float4* tile_split;
+  const int4* tile_fix;      // the FP64 path's bins in fixed point (fixed.cuh), or null: the FP64 sweep
+  const FixBlock* fix_block; // their scales, per block of 256 bins
+  const int4* fix_trig;      // the carrier's table
   const double* pref;        // [n_det][K] prefix sums of w f^-7/3
   const double* p1;          // [n_det][kNBasis][K] prefix sums of w f^-7/3 B_m (Fisher), or null
   const double* p2;          // [n_det][kNBasis (kNBasis + 1) / 2][K] ... B_m B_n, m <= n, or null

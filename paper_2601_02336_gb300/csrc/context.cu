@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "context.cuh"
+#include "fixed.cuh"
 
 using namespace sharpy;
 
@@ -68,7 +69,161 @@ __global__ void __launch_bounds__(kStageBins) tile_kernel(DevEvent ev, float4* m
   s[5 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
 }
 
+// Scales of one block of 256 bins per CTA. E_a takes 2^e with 2^e |E| <= 2^61; basis
+// function j the largest 2^b with 2^b |B| <= 2^61 for which no sum of the
+// block's products can reach 2^62 (the integer sums' high words; z is in E's
+// units / 4); the basis value 1 likewise. *bad: data that no
+// scale fits, or whose first tile lies below 2^-6 of its largest value.
+constexpr int kFixScaleThreads = 1024;
+static_assert(kFixDet * kNMom * 32 <= kFixScaleThreads, "a warp a moment");
+static_assert(kFixBins == kStageBins, "the tiles' blocks");
+__global__ void __launch_bounds__(kFixScaleThreads) fix_scale_kernel(DevEvent ev, FixBlock* out, int* bad) {
+  __shared__ double emax[2][kFixDet], bmax[2][kNBasis], sum[kFixDet][kNMom];  // [0]: first tile, [1]: block
+  const int64_t K = ev.n_bins, k0 = (int64_t)blockIdx.x * kFixBins;
+  const int64_t k1 = k0 + kFixBins < K ? k0 + kFixBins : K;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // warp w: moment (a, j) = (w / 10, w % 10) of up to 30
+  const int a = warp / kNMom, j = warp % kNMom;
+  const bool on = a < ev.n_det;
+  double em = 0.0, bm = 0.0, s = 0.0, em0 = 0.0, bm0 = 0.0;
+  bool fin = true;
+  if (on)
+    for (int64_t k = k0 + lane; k < k1; k += 32) {
+      const double2 e = ev.e64[a * K + k];
+      const double b = j < kNBasis ? fabs(ev.b64[j * K + k]) : 1.0;
+      const double l2 = hypot(e.x, e.y), lm = fmax(fabs(e.x), fabs(e.y));
+      fin = fin && isfinite(l2) && isfinite(b);
+      em = fmax(em, lm);
+      bm = fmax(bm, b);
+      if (k < k0 + 32) em0 = lm, bm0 = b;
+      s = fma(l2, b, s);
+    }
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
+    bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
+    em0 = fmax(em0, __shfl_xor_sync(0xffffffffu, em0, o));
+    bm0 = fmax(bm0, __shfl_xor_sync(0xffffffffu, bm0, o));
+    s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  fin = __all_sync(0xffffffffu, fin);
+  if (on && lane == 0) {
+    if (!fin || !isfinite(s)) atomicExch(bad, 1);
+    sum[a][j] = s;
+    if (j == 0) emax[0][a] = em0, emax[1][a] = em;
+    if (a == 0 && j < kNBasis) bmax[0][j] = bm0, bmax[1][j] = bm;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  FixBlock& fc = out[blockIdx.x];
+  int ee[kFixDet];
+  bool ok = true;
+  for (int i = 0; i < ev.n_det; ++i) {
+    const double m = emax[1][i];
+    ok = ok && (m == 0.0 || (isfinite(m) && m >= 1e-250 && emax[0][i] >= m * 0.015625));
+    ee[i] = m > 0.0 && ok ? 60 - ilogb(m) : 0;
+  }
+  for (int n = 0; n < kNMom; ++n) {
+    int be = 29 + 32;  // the basis value 1, a high limb alone
+    if (n < kNBasis) {
+      const double m = bmax[1][n];
+      ok = ok && (m == 0.0 || (isfinite(m) && m >= 1e-250 && bmax[0][n] >= m * 0.015625));
+      be = m > 0.0 && ok ? 60 - ilogb(m) : 0;
+    }
+    for (int i = 0; i < ev.n_det; ++i)
+      if (ok && sum[i][n] > 0.0) be = min(be, 127 - ee[i] - ilogb(sum[i][n]));
+    if (n == kNBasis) {
+      ok = ok && be >= 32;
+      fc.one = ok ? 1 << (be - 32) : 0;
+    }
+    for (int i = 0; i < ev.n_det; ++i) {
+      ok = ok && abs(66 - ee[i] - be) <= 1000;
+      fc.scale[i * kNMom + n] = ldexp(1.0, ok ? 66 - ee[i] - be : 0);
+    }
+    fc.be[n] = be;
+  }
+  for (int i = 0; i < ev.n_det; ++i) fc.ee[i] = ee[i];
+  if (!ok) atomicExch(bad, 1);
+}
+
+// One CTA per block of kStageBins bins, one thread per bin: the bin's
+// fixed-point quads (zeros past the last bin).
+__global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const FixBlock* fc, const int* bad, int4* out) {
+  if (*bad) return;
+  const int64_t K = ev.n_bins, k = (int64_t)blockIdx.x * kStageBins + threadIdx.x;
+  const bool in = k < K;
+  const FixBlock& c = fc[k / kFixBins];
+  int4* t = out + k / kTileBins * (kFixQuads * kTileBins) + k % kTileBins;
+  for (int j = 0; j < kNBasis; ++j) {
+    const double b = in ? ev.b64[j * K + k] : 0.0;
+    const Limbs l = fix_limbs_neg((int64_t)rint(ldexp(b, c.be[j])));
+    t[j * kTileBins] = make_int4(__double2loint(b), __double2hiint(b), l.h, l.l);
+  }
+  for (int a = 0; a < kFixDet; ++a) {
+    const double2 e = in && a < ev.n_det ? ev.e64[a * K + k] : make_double2(0.0, 0.0);
+    const int s = a < ev.n_det ? c.ee[a] : 0;
+    const Limbs x = fix_limbs_neg((int64_t)rint(ldexp(e.x, s))), y = fix_limbs_neg((int64_t)rint(ldexp(e.y, s)));
+    t[(kNBasis + a) * kTileBins] = make_int4(x.h, x.l, y.h, y.l);
+  }
+}
+
 }  // namespace sharpy
+
+// The carrier's table, cos and sin of 2 pi i / 1024 to 2^-62 (from the first
+// octant, where long double has the bits for it on every host).
+static const int4* fix_trig_host() {
+  static const std::vector<int4> t = [] {
+    std::vector<int4> v(kFixTrig);
+    const long double w = 6.283185307179586476925286766559L / kFixTrig;
+    for (int i = 0; i < kFixTrig; ++i) {
+      const int q = i * 4 / kFixTrig, r = i % (kFixTrig / 4);  // quadrant, place in it
+      const bool swap = r > kFixTrig / 8;
+      const long double x = w * (swap ? kFixTrig / 4 - r : r);
+      const int64_t a = (int64_t)std::rint(std::ldexp(swap ? std::sin(x) : std::cos(x), 62));
+      const int64_t b = (int64_t)std::rint(std::ldexp(swap ? std::cos(x) : std::sin(x), 62));
+      const Limbs c = fix_limbs_neg(q == 0 ? a : q == 1 ? -b : q == 2 ? -a : b);
+      const Limbs s = fix_limbs_neg(q == 0 ? b : q == 1 ? a : q == 2 ? -b : -a);
+      v[i] = make_int4(c.h, c.l, s.h, s.l);
+    }
+    return v;
+  }();
+  return t.data();
+}
+
+// The fixed-point tables of the FP64 path, built with every data set; without
+// them (memory, too many bins, data that no scale fits) the FP64 sweep runs.
+static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
+  DevEvent& ev = c->ev;
+  ev.tile_fix = nullptr;
+  ev.fix_block = nullptr;
+  ev.fix_trig = nullptr;
+  if (ev.n_bins > kFixMaxBins || ev.n_det > kFixDet) return cudaSuccess;
+  const size_t tiles = (size_t)blocks * kStageBins * kFixQuads;
+  const size_t scales = (size_t)((ev.n_bins + kFixBins - 1) / kFixBins);
+  if (!c->d_fix) {
+    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig) * sizeof(int4) + (size_t)blocks * sizeof(FixBlock) + sizeof(int)) != cudaSuccess) {
+      c->d_fix = nullptr;
+      (void)cudaGetLastError();
+      return cudaSuccess;
+    }
+    const cudaError_t e = cudaMemcpy(c->d_fix + tiles, fix_trig_host(), kFixTrig * sizeof(int4), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) return e;
+  }
+  FixBlock* fc = reinterpret_cast<FixBlock*>(c->d_fix + tiles + kFixTrig);
+  int* bad = reinterpret_cast<int*>(fc + blocks);
+  cudaError_t e = cudaMemset(bad, 0, sizeof(int));
+  if (e != cudaSuccess) return e;
+  fix_scale_kernel<<<(unsigned)blocks, kFixScaleThreads>>>(ev, fc, bad);
+  fix_tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, fc, bad, c->d_fix);
+  int b = 1;
+  e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaMemcpy(&b, bad, sizeof(int), cudaMemcpyDeviceToHost);
+  if (e != cudaSuccess || b) return e;
+  ev.tile_fix = c->d_fix;
+  ev.fix_block = fc;
+  ev.fix_trig = c->d_fix + tiles;
+  return cudaSuccess;
+}
 
 static void free_event(sharpy_ctx* c) {
   cudaFree(c->d_f);
@@ -78,7 +233,9 @@ static void free_event(sharpy_ctx* c) {
   cudaFree(c->d_p1);
   cudaFree(c->d_p2);
   cudaFree(c->d_tile);
+  cudaFree(c->d_fix);
   c->d_tile = nullptr;
+  c->d_fix = nullptr;
   c->d_p1 = c->d_p2 = nullptr;
   c->ev.p1 = c->ev.p2 = nullptr;
   c->d_f = c->d_b64 = c->d_pref = nullptr;
@@ -302,7 +459,7 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   // the sweeps' tiles (rebuilt with every data set: they hold E)
   float4* split = c->d_tile + blocks * (stage_bytes(false) / 16);
   tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, c->d_tile, split);
-  if (cudaGetLastError() != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+  if (cudaGetLastError() != cudaSuccess || build_fixed(c, blocks) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
     free_event(c);
     return SHARPY_ECUDA;
   }

@@ -59,7 +59,7 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
       double v[FS::KEEP];
       if (PREC == SHARPY_FP64) {
         if (live) {
-          fp64_stream<GRAD, NDET>(ev, sc[pl], st, v);
+          wide_stream<GRAD, NDET>(ev, sc[pl], st, v);
         } else {
 #pragma unroll
           for (int t = 0; t < FS::KEEP; ++t) v[t] = 0.0;

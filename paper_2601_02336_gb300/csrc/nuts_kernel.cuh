@@ -945,7 +945,7 @@ __global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
         }
         double v[FS::KEEP];
         if constexpr (PREC == SHARPY_FP64) {
-          fp64_stream<true, NDET>(A.ev, sc[slot], st, v);
+          wide_stream<true, NDET>(A.ev, sc[slot], st, v);
         } else {
           float hi[FS::KEEP], lo[FS::KEEP];
           mixed_stream<true, NDET, PREC == SHARPY_MIXED_SPLIT>(A.ev, sc[slot], st, hi, lo);

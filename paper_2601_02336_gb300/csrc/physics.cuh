@@ -557,7 +557,6 @@ __device__ __forceinline__ void prologue_cta(int warp, int lane, int n, const De
 }
 
 // Moments layout: mom[a][j][re/im], j = 0..8 basis (8 = f), j = 9 plain sum Z.
-constexpr int kNMom = kNBasis + 1;
 
 // ln L (FP64 total) and d lnL / d(physical parameters) from the moments.
 // The gradient is contracted on the amplitude-scaled moments A0 Z, A0 Y_j and

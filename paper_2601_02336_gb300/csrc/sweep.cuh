@@ -7,7 +7,10 @@
 // carrier e^{-i Psi}, multiplies the pre-whitened data E_ak and accumulates
 // Z_a (and, for the gradient, Y_aj = sum z B_j).
 //
-//   SHARPY_FP64  : FP64 throughout; reduction Psi - rint(Psi); sincospi.
+//   SHARPY_FP64  : the phase in FP64; carrier, data product and moments in
+//                  64-bit fixed point (fixed.cuh: errors below FP64's), or, for
+//                  data that it does not fit, FP64 throughout (reduction
+//                  Psi - rint(Psi); sincospi).
 //   SHARPY_MIXED_SPLIT : as SHARPY_MIXED, but the phase polynomial is built
 //                  from hi/lo FP32 splits of alpha_j, tau_a and B_j(f_k):
 //                  each product's integer turns are removed exactly (FMA error
@@ -26,17 +29,19 @@
 //                  into compensated FP32 outer accumulators (blocked pairwise
 //                  summation).
 #pragma once
+#include "fixed.cuh"
 #include "physics.cuh"
 
 namespace sharpy {
 
-constexpr int kFlush = 64;  // lane iterations per FP32 block
+constexpr int kFlush = 64;  // lane iterations per block
 // Long sweeps are cut into chunks of kFlush lane iterations (2048 bins) dealt
 // to kStreams streams (chunk c to stream c mod kStreams); a stream's result
 // does not depend on which warp computes it, and streams are merged in a fixed
 // order, so any number of warps per particle gives the same moments.
 constexpr int kChunkBins = kFlush * 32;
 constexpr int kStreams = 8;
+static_assert(kChunkBins % kFixBins == 0, "chunks are whole blocks of the fixed-point scales");
 
 template <int NDET, bool GRAD>
 struct MomCount {
@@ -475,6 +480,91 @@ __device__ void sweep_mixed(const DevEvent& ev, const SweepCoef& sc, float* mom)
   }
 }
 
+// One stream of the FP64 path in fixed point (chunks c = s, s + kStreams, ...
+// of 2048 bins below k_ISCO): the integer sums of each block of 256 bins go
+// through the warp reduce-scatter exactly (~500 instructions against the
+// block's ~4000), are rounded to FP64 once and added to the stream's; lane l
+// holds its sums in v_out. Returns whether the stream had any bin.
+// Per bin and detector 4 FP64 instructions and ~170 integer ones against ~50
+// FP64 ones of fp64_stream (60 cycles each): see fixed.cuh.
+template <bool GRAD, int NDET>
+__device__ bool fixed_stream(const DevEvent& ev, const SweepCoef& sc, int s, double* v_out) {
+  constexpr int NACC = MomCount<NDET, GRAD>::value;
+  using F = FlushShape<NACC>;
+  const int lane = threadIdx.x & 31;
+  double al[kNPn];
+#pragma unroll
+  for (int j = 0; j < kNPn; ++j) al[j] = sc.alpha[j];
+#pragma unroll
+  for (int t = 0; t < F::KEEP; ++t) v_out[t] = 0.0;
+  const int kend = sc.kisco;
+  uint32_t top = 0;  // largest exponent of a phase: a non-finite one has no fraction
+  bool any = false;
+  // blocks of the chunks s, s + kStreams, ...
+  constexpr int kPer = kChunkBins / kFixBins;
+#pragma unroll 1
+  for (int g = s * kPer; g * kFixBins <= kend; g += (g % kPer == kPer - 1 ? (kStreams - 1) * kPer : 0) + 1) {
+    any = true;
+    int64_t acc[NACC];
+#pragma unroll
+    for (int i = 0; i < NACC; ++i) acc[i] = 0;
+    const FixBlock* fb = ev.fix_block + g;
+    const int one = __ldg(&fb->one);
+    const int kstop = min(kend, g * kFixBins + kFixBins - 1);
+    const int4* at = ev.tile_fix + (int64_t)g * (kFixBins * kFixQuads) + lane;
+#pragma unroll 1
+    for (int k = g * kFixBins + lane; k <= kstop; k += 32, at += kFixQuads * kTileBins) {
+      double S = sc.c0, f = 0.0;
+      int bh[kNBasis], bl[kNBasis];
+#pragma unroll
+      for (int j = 0; j < kNBasis; ++j) {
+        const int4 q = __ldg(at + j * kTileBins);
+        const double b = __hiloint2double(q.y, q.x);
+        bh[j] = q.z;
+        bl[j] = q.w;
+        if (j < kNPn)
+          S = fma(al[j < kNPn ? j : 0], b, S);
+        else
+          f = b;
+      }
+#pragma unroll
+      for (int a = 0; a < NDET; ++a) {
+        const double P = fma(f, sc.tau[a], S);
+        top = max(top, (uint32_t)__double2hiint(P) & 0x7ff00000u);
+        const uint64_t u = fix_frac(P);
+        int64_t zr, zi;
+        fix_carrier(u, __ldg(at + (kNBasis + a) * kTileBins), __ldg(ev.fix_trig + fix_index(u)), &zr, &zi);
+        const Limbs r = fix_limbs(zr), i = fix_limbs(zi);
+        if (GRAD) {
+#pragma unroll
+          for (int j = 0; j < kNBasis; ++j) {
+            int64_t* m = acc + (a * kNMom + j) * 2;
+            m[0] = fix_moment(r, bh[j], bl[j], m[0]);
+            m[1] = fix_moment(i, bh[j], bl[j], m[1]);
+          }
+        }
+        int64_t* m = acc + (GRAD ? (a * kNMom + 9) * 2 : a * 2);
+        m[0] = fix_moment(r, one, 0, m[0]);
+        m[1] = fix_moment(i, one, 0, m[1]);
+      }
+    }
+    int64_t v[F::NP];
+#pragma unroll
+    for (int i = 0; i < F::NP; ++i) v[i] = i < NACC ? acc[i] : 0;
+    ReduceScatter<F::NP, 16, int64_t>::run(v, lane);
+#pragma unroll
+    for (int t = 0; t < F::KEEP; ++t) {
+      const int i = F::index(lane, t);
+      if (i < NACC) v_out[t] = fma((double)v[t], __ldg(fb->scale + (GRAD ? i / 2 : i / 2 * kNMom + 9)), v_out[t]);
+    }
+  }
+  if (__any_sync(0xffffffffu, top >= 0x7ff00000u)) {
+#pragma unroll
+    for (int t = 0; t < F::KEEP; ++t) v_out[t] = NAN;
+  }
+  return any;
+}
+
 // One stream of the FP64 sweep (chunks c = s, s + kStreams, ... of 2048 bins
 // below k_ISCO): per-lane FP64 sums, then the warp reduce-scatter (the same
 // pairing as a butterfly sum per moment, with NP/2 + NP/4 + ... FP64 adds per
@@ -540,6 +630,12 @@ __device__ bool fp64_stream(const DevEvent& ev, const SweepCoef& sc, int s, doub
   return any;
 }
 
+// One stream of the FP64 path, in the arithmetic that the event's data allow.
+template <bool GRAD, int NDET>
+__device__ bool wide_stream(const DevEvent& ev, const SweepCoef& sc, int s, double* v_out) {
+  return ev.tile_fix ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
+}
+
 // FP64 moments of one particle on one warp; streams as in sweep_mixed (a
 // sweep below 2048 bins is its single stream).
 template <bool GRAD, int NDET>
@@ -549,12 +645,12 @@ __device__ void sweep_fp64(const DevEvent& ev, const SweepCoef& sc, double* mom)
   const int lane = threadIdx.x & 31;
   double v[F::KEEP], tot[F::KEEP];
   if (sc.kisco < kChunkBins) {
-    fp64_stream<GRAD, NDET>(ev, sc, 0, tot);
+    wide_stream<GRAD, NDET>(ev, sc, 0, tot);
   } else {
 #pragma unroll
     for (int t = 0; t < F::KEEP; ++t) tot[t] = 0.0;
     for (int st = 0; st < kStreams; ++st) {
-      if (!fp64_stream<GRAD, NDET>(ev, sc, st, v)) break;
+      if (!wide_stream<GRAD, NDET>(ev, sc, st, v)) break;
 #pragma unroll
       for (int t = 0; t < F::KEEP; ++t) tot[t] += v[t];
     }

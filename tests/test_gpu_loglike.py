@@ -342,3 +342,39 @@ def test_loglike_tile_edges(name, n_bins):
             err = np.linalg.norm((g.cpu().numpy() - ref_g) * wid, axis=1)
             assert np.all(err <= np.maximum(1e-4 * norm, 1e-3)), (prec, split)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("n_bins,outlier", [(1, 0), (31, 0), (32, 0), (33, 0), (255, 0), (256, 0), (257, 0), (2047, 0),
+                                            (2048, 0), (2049, 0), (600, 4), (600, 12), (600, 40)])
+@pytest.mark.parametrize("name", ["tiny", "bbh11"])
+def test_loglike_fp64_block_edges(name, n_bins, outlier):
+    """The FP64 path's fixed-point bins are scaled per block of 256, in chunks of 2048: segments around each edge agree
+    with the oracle within the path's bounds (ln L 1e-7 + 1e-10 |ln L|, the gradient 1e-8 of its norm in prior widths,
+    or 1e-6 where the norm is below the ln L bound's scale). One bin scaled up by 2^outlier: the smaller factors widen
+    its block's range, beyond 2^6 the event takes the FP64 sweep. One and three detectors, with and without the
+    gradient, on one warp and on eight warps a vector, which agree bit for bit."""
+    G.require_gpu()
+    w = inputs.WORKLOADS[name]()
+    w.n_bins = n_bins
+    ev, ctx, th_inj, data = G.event_pair(w, seed=0)
+    if outlier:
+        data = data.copy()
+        data[:, 300] *= 2.0 ** outlier
+        ev = helpers.oracle_event(w, data=data)
+        ctx.set_data(data, inputs.psd_array(w), w.f_min, w.df, inputs.detectors(w))
+    th = np.vstack([inputs.prior_draws(w, 6, 51), inputs.ball(w, th_inj, 5, 52)])
+    ref_l, ref_g = oracle.loglike(helpers.oracle_model(w), ev, th)
+    wid = G.width(w)
+    norm = np.linalg.norm(ref_g * wid, axis=1)
+    out = []
+    for split in (1, 8):
+        ctx.set_loglike_split(split)
+        l, g = ctx.loglike_grad(G.to_dev(th), "fp64")
+        l0, _ = ctx.loglike_grad(G.to_dev(th), "fp64", grad=False)
+        out.append((l, g, l0))
+        for x in (l, l0):
+            assert np.all(np.abs(x.cpu().numpy() - ref_l) <= 1e-7 + 1e-10 * np.abs(ref_l)), split
+        err = np.linalg.norm((g.cpu().numpy() - ref_g) * wid, axis=1)
+        assert np.all(err <= np.maximum(1e-8 * norm, 1e-6)), split
+    assert all(torch.equal(a, b) for a, b in zip(*out))
+    assert ctx.status() == 0
