@@ -86,6 +86,25 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
       }
     }
   }
+  if constexpr (PREC == SHARPY_FP64) {
+    // the particle's first warp, which wrote its moments: lanes (detector, direction)
+    __shared__ double gph[PPC][SHARPY_NPHYS];
+    if (r != 0 || p >= n) return;
+    __syncwarp();
+    double l = NAN;
+    const bool ok = sc[pl].ok != 0;
+    if (ok) epilogue_lanes<GRAD, 16>(ev, sc[pl], ec[pl], mom[pl], lane & 15, 0xffffffffu, &l, gph[pl]);
+    __syncwarp();
+    bool fin = isfinite(l);
+    if (lane == 0) lnl[p] = l;
+    if (GRAD && lane < D) {
+      const double g = ok ? gph[pl][m.phys[lane]] : NAN;
+      grad[p * D + lane] = g;
+      fin = fin && isfinite(g);
+    }
+    if (!fin) set_status(status, SHARPY_ENONFINITE);
+    return;
+  }
   __syncthreads();
   if (warp == 0 && lane < PPC) {
     int64_t q = base + lane;

@@ -657,6 +657,7 @@ struct NutsSmem {
   SweepCoef sc[SLOTS];
   EpiCoef<DT> ec[SLOTS];
   MT mom[SLOTS][NDET * kNMom * 2];
+  double gph[PREC == SHARPY_FP64 ? SLOTS : 1][SHARPY_NPHYS];  // FP64 path: the epilogues' gradients
 };
 
 // CTAs per SM the registers are held to: 16 warps an SM at 128 registers (a
@@ -858,9 +859,36 @@ __global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
     }
     __syncthreads();
     if (!S.alive) break;
-    // (A) prologues (GW models; lane = slot): the phase on the control warp, the
-    // amplitude and the sky on its neighbour, on another sub-partition
-    if (gw && (warp == cw || warp == (cw ^ 1)) && lane < SLOTS && S.pending[lane]) {
+    // (A) prologues. FP64 path: an instruction takes 60 cycles of the pipe
+    // however many lanes are on, so a slot's phase goes to four lanes, one
+    // direction each, its sky to a lane a detector; tasks of eight slots and the
+    // amplitudes, longest first, one a warp in turn. Otherwise lane = slot: the
+    // phase on the control warp, the amplitude and the sky on its neighbour, on
+    // another sub-partition.
+    if constexpr (PREC == SHARPY_FP64) {
+      if (gw) {
+        const unsigned pm = __ballot_sync(0xffffffffu, lane < SLOTS && S.pending[lane]);
+        const int np = __popc(pm), n8 = (np + 7) / 8;
+        for (int task = (warp - cw) & (W - 1); task < 2 * n8 + 1; task += W) {
+          const int kind = task < n8 ? 0 : task < 2 * n8 ? 1 : 2;  // phase, sky, amplitude
+          const int i = kind == 2 ? lane : (task - kind * n8) * 8 + lane / 4, k = lane & 3;
+          if (i >= np || (kind == 1 && k >= A.ev.n_det)) continue;
+          unsigned left = pm;
+          for (int j = 0; j < i; ++j) left &= left - 1;
+          const int slot = __ffs(left) - 1;
+          double x[kMaxDim];
+          for (int d = 0; d < D; ++d) x[d] = S.pos[P_N][slot][d];
+          if (kind == 0)
+            prologue_phase<DT, true, false, 1>(A.m, A.ev, x, sc[slot], ec[slot], k);
+          else if (kind == 1)
+            prologue_sky_one<DT, true>(A.m, A.ev, x, k, sc[slot], ec[slot]);
+          else
+            prologue_amp<DT, true>(A.m, x, ec[slot]);
+        }
+        if (SLOTS > 8) __syncthreads();  // the order below reads every slot's k_ISCO
+        __syncwarp();
+      }
+    } else if (gw && (warp == cw || warp == (cw ^ 1)) && lane < SLOTS && S.pending[lane]) {
       double x[kMaxDim];
       for (int i = 0; i < D; ++i) x[i] = S.pos[P_N][lane][i];
       if (warp == cw) {
@@ -982,10 +1010,17 @@ __global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
 #pragma unroll
       for (int k = 0; k < DPL; ++k) x[k] = nu.has(k) ? nu.X(P_N, nu.dim(k)) : 0.0;
       if (gw) {
-        DT gph[SHARPY_NPHYS];
+        DT gown[PREC == SHARPY_FP64 ? 1 : SHARPY_NPHYS];
+        const DT* gph = gown;
         sl.lnl_new = NAN;
         if (sc[cs].ok) {
-          epilogue<DT, true>(A.ev, sc[cs], ec[cs], mom[cs], &sl.lnl_new, gph);
+          if constexpr (PREC == SHARPY_FP64) {
+            epilogue_lanes<true, G>(A.ev, sc[cs], ec[cs], mom[cs], tg, gmask, &sl.lnl_new, SM.gph[cs]);
+            gph = SM.gph[cs];
+            __syncwarp(gmask);
+          } else {
+            epilogue<DT, true>(A.ev, sc[cs], ec[cs], mom[cs], &sl.lnl_new, gown);
+          }
           sl.st_bins += (long long)(sc[cs].kisco + 1) * A.ev.n_det;
         }
 #pragma unroll

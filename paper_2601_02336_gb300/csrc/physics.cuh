@@ -27,26 +27,27 @@
 
 namespace sharpy {
 
-// Value with derivatives along four directions. The value is FP64 (DT =
+// Value with derivatives along N directions (all four, or one where a lane
+// carries one of them). The value is FP64 (DT =
 // double) or double-float (DT = float); for DT = float an FP32 shadow of the
 // value feeds the derivative arithmetic, so derivatives need neither FP64
 // operations nor conversions.
-template <class DT>
+template <class DT, int N = 4>
 struct I4;
 
-template <>
-struct I4<double> {
+template <int N>
+struct I4<double, N> {
   double v;
-  double d[4];
+  double d[N];
   __device__ __forceinline__ double f() const { return v; }
   __device__ __forceinline__ void setf(double) {}
 };
 
-template <>
-struct I4<float> {
+template <int N>
+struct I4<float, N> {
   DF v;
   float vf;
-  float d[4];
+  float d[N];
   __device__ __forceinline__ float f() const { return vf; }
   __device__ __forceinline__ void setf(float x) { vf = x; }
 };
@@ -68,94 +69,97 @@ __device__ __forceinline__ auto vval(double x) {
     return df_from(x);
 }
 
-template <class DT>
-__device__ __forceinline__ I4<DT> iconst(double x) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> iconst(double x) {
+  I4<DT, N> r;
   r.v = vval<DT>(x);
   r.setf((DT)x);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = DT(0);
+  for (int i = 0; i < N; ++i) r.d[i] = DT(0);
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> ivar(double x, int k) {
-  I4<DT> r = iconst<DT>(x);
-  r.d[k] = DT(1);
+// variable k; the directions start at `first`
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> ivar(double x, int k, int first) {
+  I4<DT, N> r = iconst<DT, N>(x);
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (first + i == k) r.d[i] = DT(1);
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> operator+(const I4<DT>& a, const I4<DT>& b) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> operator+(const I4<DT, N>& a, const I4<DT, N>& b) {
+  I4<DT, N> r;
   r.v = a.v + b.v;
   r.setf(a.f() + b.f());
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = a.d[i] + b.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = a.d[i] + b.d[i];
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> operator-(const I4<DT>& a, const I4<DT>& b) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> operator-(const I4<DT, N>& a, const I4<DT, N>& b) {
+  I4<DT, N> r;
   r.v = a.v - b.v;
   r.setf(a.f() - b.f());
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = a.d[i] - b.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = a.d[i] - b.d[i];
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> operator*(const I4<DT>& a, const I4<DT>& b) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> operator*(const I4<DT, N>& a, const I4<DT, N>& b) {
+  I4<DT, N> r;
   r.v = a.v * b.v;
   r.setf(a.f() * b.f());
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = a.d[i] * b.f() + a.f() * b.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = a.d[i] * b.f() + a.f() * b.d[i];
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> operator*(double s, const I4<DT>& a) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> operator*(double s, const I4<DT, N>& a) {
+  I4<DT, N> r;
   r.v = s * a.v;
   r.setf((DT)s * a.f());
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = (DT)s * a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = (DT)s * a.d[i];
   return r;
 }
-template <class DT>
-__device__ __forceinline__ I4<DT> operator+(double s, const I4<DT>& a) {
-  I4<DT> r = a;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> operator+(double s, const I4<DT, N>& a) {
+  I4<DT, N> r = a;
   r.v = s + a.v;
   r.setf((DT)s + a.f());
   return r;
 }
 // 1 / a
-template <class DT>
-__device__ __forceinline__ I4<DT> recip(const I4<DT>& a) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> recip(const I4<DT, N>& a) {
+  I4<DT, N> r;
   r.v = vrecip(a.v);
   r.setf(vlow<DT>(r.v));
   const DT g = -r.f() * r.f();
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = g * a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = g * a.d[i];
   return r;
 }
 // ln a
-template <class DT>
-__device__ __forceinline__ I4<DT> ilog(const I4<DT>& a) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> ilog(const I4<DT, N>& a) {
+  I4<DT, N> r;
   r.v = log(a.v);
   r.setf((DT)r.v);
   const DT g = DT(1) / a.f();
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = g * a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = g * a.d[i];
   return r;
 }
 // e^a
-template <class DT>
-__device__ __forceinline__ I4<DT> iexp(const I4<DT>& a) {
-  I4<DT> r;
+template <class DT, int N>
+__device__ __forceinline__ I4<DT, N> iexp(const I4<DT, N>& a) {
+  I4<DT, N> r;
   r.v = exp(a.v);
   r.setf((DT)r.v);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) r.d[i] = r.f() * a.d[i];
+  for (int i = 0; i < N; ++i) r.d[i] = r.f() * a.d[i];
   return r;
 }
 
@@ -205,8 +209,9 @@ __device__ __forceinline__ void to_physical(const DevModel& m, const double* th,
 // u = c v^14, ln u by the double-float logarithm (it sets the constant and
 // 3PN phase terms, which need ~1e-10). Derivatives from
 // d ln u = (d Mc / Mc - 3/5 d eta / eta) / 3.
-__device__ __forceinline__ void u_mixed(const I4<float>& mcv, const I4<float>& eta, const I4<float>& ieta,
-                                        I4<float>& u, I4<float>& ui, I4<float>& lnu) {
+template <int N>
+__device__ __forceinline__ void u_mixed(const I4<float, N>& mcv, const I4<float, N>& eta, const I4<float, N>& ieta,
+                                        I4<float, N>& u, I4<float, N>& ui, I4<float, N>& lnu) {
   const DF p = (kPi * kTsun) * mcv.v;
   const DF p2 = p * p;
   const DF ie = ieta.v;
@@ -229,30 +234,32 @@ __device__ __forceinline__ void u_mixed(const I4<float>& mcv, const I4<float>& e
   ui.vf = v.hi;
   const float imc = 1.0f / mcv.vf, ieta_f = 1.0f / eta.vf;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
+  for (int i = 0; i < N; ++i) {
     lnu.d[i] = (1.0f / 3.0f) * (mcv.d[i] * imc - 0.6f * eta.d[i] * ieta_f);
     u.d[i] = u.vf * lnu.d[i];
     ui.d[i] = -ui.vf * lnu.d[i];
   }
 }
 
-// TaylorF2 phase coefficients in turns and their Jacobian w.r.t. (Mc, q, chi1, chi2).
+// TaylorF2 phase coefficients in turns and their Jacobian w.r.t. (Mc, q, chi1, chi2),
+// of it the N directions from `first`.
 // FP64 path: ln eta, ln Mc and one exponential (u) in FP64; mixed path: u_mixed.
-template <class DT>
-__device__ void pn_coefficients(const double* ph, I4<DT>* alpha, I4<DT>& cpn, double& mtot, double& fisco) {
-  const I4<DT> mc = ivar<DT>(ph[SHARPY_MC], 0);
-  const I4<DT> q = ivar<DT>(ph[SHARPY_Q], 1);
-  const I4<DT> c1 = ivar<DT>(ph[SHARPY_CHI1], 2);
-  const I4<DT> c2 = ivar<DT>(ph[SHARPY_CHI2], 3);
-  const I4<DT> onepq = 1.0 + q;
-  const I4<DT> m1 = recip(onepq);  // m1 / M
-  const I4<DT> m2 = q * m1;        // m2 / M
-  const I4<DT> eta = m1 * m2;
-  const I4<DT> delta = m1 - m2;
-  const I4<DT> iq = recip(q);
-  const I4<DT> ieta = onepq * onepq * iq;  // 1 / eta = (1+q)^2 / q
+template <class DT, int N>
+__device__ void pn_coefficients(const double* ph, int first, I4<DT, N>* alpha, I4<DT, N>& cpn, double& mtot,
+                                double& fisco) {
+  const I4<DT, N> mc = ivar<DT, N>(ph[SHARPY_MC], 0, first);
+  const I4<DT, N> q = ivar<DT, N>(ph[SHARPY_Q], 1, first);
+  const I4<DT, N> c1 = ivar<DT, N>(ph[SHARPY_CHI1], 2, first);
+  const I4<DT, N> c2 = ivar<DT, N>(ph[SHARPY_CHI2], 3, first);
+  const I4<DT, N> onepq = 1.0 + q;
+  const I4<DT, N> m1 = recip(onepq);  // m1 / M
+  const I4<DT, N> m2 = q * m1;        // m2 / M
+  const I4<DT, N> eta = m1 * m2;
+  const I4<DT, N> delta = m1 - m2;
+  const I4<DT, N> iq = recip(q);
+  const I4<DT, N> ieta = onepq * onepq * iq;  // 1 / eta = (1+q)^2 / q
   // ln u = (ln(pi Tsun) + ln Mc - 3/5 ln eta) / 3, v = u f^(1/3), M = u^3 / (pi Tsun)
-  I4<DT> lnu, u, ui;
+  I4<DT, N> lnu, u, ui;
   if constexpr (std::is_same<DT, double>::value) {
     lnu = (1.0 / 3.0) * ((-11.076356701842613) + (ilog(mc) + (-0.6) * ilog(eta)));
     u = iexp(lnu);
@@ -264,29 +271,29 @@ __device__ void pn_coefficients(const double* ph, I4<DT>* alpha, I4<DT>& cpn, do
     mtot = 0.0;  // not needed: f_ISCO from 1/u directly
     fisco = df_to_double((1.0 / 14.696938456699069) * (ui.v * ui.v * ui.v));  // 1 / (6^(3/2) u^3)
   }
-  const I4<DT> chis = 0.5 * (c1 + c2);
-  const I4<DT> chia = 0.5 * (c1 - c2);
-  const I4<DT> eta2 = eta * eta;
+  const I4<DT, N> chis = 0.5 * (c1 + c2);
+  const I4<DT, N> chia = 0.5 * (c1 - c2);
+  const I4<DT, N> eta2 = eta * eta;
   // spin-orbit (1.5PN, 2.5PN) and spin-spin (2PN) combinations
-  const I4<DT> beta = ((113.0 / 12.0) + (-19.0 / 3.0) * eta) * chis + (113.0 / 12.0) * (delta * chia);
-  const I4<DT> gam = ((732985.0 / 2268.0) + ((-24260.0 / 81.0) * eta + (-340.0 / 9.0) * eta2)) * chis +
+  const I4<DT, N> beta = ((113.0 / 12.0) + (-19.0 / 3.0) * eta) * chis + (113.0 / 12.0) * (delta * chia);
+  const I4<DT, N> gam = ((732985.0 / 2268.0) + ((-24260.0 / 81.0) * eta + (-340.0 / 9.0) * eta2)) * chis +
                      ((732985.0 / 2268.0) + (140.0 / 9.0) * eta) * (delta * chia);
-  const I4<DT> sig =
+  const I4<DT, N> sig =
       (79.0 / 8.0) * (eta * (c1 * c2)) + (81.0 / 16.0) * (m1 * m1 * c1 * c1 + m2 * m2 * c2 * c2);
-  const I4<DT> p2 = (3715.0 / 756.0) + (55.0 / 9.0) * eta;
-  const I4<DT> p3 = (-16.0 * kPi) + 4.0 * beta;
-  const I4<DT> p4 =
+  const I4<DT, N> p2 = (3715.0 / 756.0) + (55.0 / 9.0) * eta;
+  const I4<DT, N> p3 = (-16.0 * kPi) + 4.0 * beta;
+  const I4<DT, N> p4 =
       (15293365.0 / 508032.0) + ((27145.0 / 504.0) * eta + (3085.0 / 72.0) * eta2 + (-10.0) * sig);
-  const I4<DT> p5 = (kPi * 38645.0 / 756.0) + ((-kPi * 65.0 / 9.0) * eta - gam);
-  const I4<DT> p6 =
+  const I4<DT, N> p5 = (kPi * 38645.0 / 756.0) + ((-kPi * 65.0 / 9.0) * eta - gam);
+  const I4<DT, N> p6 =
       (11583231236531.0 / 4694215680.0 - 640.0 / 3.0 * kPi * kPi - 6848.0 / 21.0 * kEulerGamma) +
       ((-15737765635.0 / 3048192.0 + 2255.0 / 12.0 * kPi * kPi) * eta + (76055.0 / 1728.0) * eta2 +
        (-127825.0 / 1296.0) * (eta2 * eta));
-  const I4<DT> p7 = kPi * ((77096675.0 / 254016.0) + ((378515.0 / 1512.0) * eta + (-74045.0 / 756.0) * eta2));
+  const I4<DT, N> p7 = kPi * ((77096675.0 / 254016.0) + ((378515.0 / 1512.0) * eta + (-74045.0 / 756.0) * eta2));
   // 3 / (128 eta) in turns
-  const I4<DT> nt = (3.0 / (128.0 * kTwoPi)) * ieta;
-  const I4<DT> ui2 = ui * ui;
-  const I4<DT> ui3 = ui2 * ui;
+  const I4<DT, N> nt = (3.0 / (128.0 * kTwoPi)) * ieta;
+  const I4<DT, N> ui2 = ui * ui;
+  const I4<DT, N> ui3 = ui2 * ui;
   alpha[0] = nt * (ui3 * ui2);  // x^5
   alpha[1] = nt * (p2 * ui3);   // x^3
   alpha[2] = nt * (p3 * ui2);   // x^2
@@ -398,33 +405,38 @@ __device__ __forceinline__ bool phys_ok(const double* ph) {
 // once: the phase (alpha, c0, k_ISCO, ok and their Jacobians), the amplitude,
 // and the sky of each detector (responses C_a, delays tau_a and theirs). None
 // reads what another writes.
-template <class DT, bool GRAD, bool SPLIT = false>
+// N < 4: this lane has the N directions from `first` of the Jacobian (lanes of
+// one particle store their own, the first lane what they share).
+template <class DT, bool GRAD, bool SPLIT = false, int N = 4>
 __device__ void prologue_phase(const DevModel& m, const DevEvent& ev, const double* th, SweepCoef& sc,
-                               EpiCoef<DT>& ec) {
+                               EpiCoef<DT>& ec, int first = 0) {
   double ph[SHARPY_NPHYS];
   to_physical(m, th, ph);
-  sc.ok = phys_ok(ph) ? 1 : 0;
-  if (!sc.ok) {
-    sc.kisco = -1;
-    return;
+  const bool ok = phys_ok(ph), lead = N == 4 || first == 0;
+  if (lead) {
+    sc.ok = ok ? 1 : 0;
+    if (!ok) sc.kisco = -1;
   }
-  I4<DT> alpha[kNPn], cpn;
+  if (!ok) return;
+  I4<DT, N> alpha[kNPn], cpn;
   double mtot, fisco;
-  pn_coefficients<DT>(ph, alpha, cpn, mtot, fisco);
+  pn_coefficients<DT, N>(ph, first, alpha, cpn, mtot, fisco);
+  if (GRAD) {
+#pragma unroll
+    for (int j = 0; j < kNPn; ++j)
+#pragma unroll
+      for (int i = 0; i < N; ++i) ec.dalpha[j][first + i] = alpha[j].d[i];
+#pragma unroll
+    for (int i = 0; i < N; ++i) ec.dc0[first + i] = cpn.d[i];
+  }
+  if (!lead) return;
   // the mixed sweep reads the four large terms' coefficients in FP64 and the
   // others as FP32 pairs: only the four get an FP64 copy there
   constexpr bool kAllF64 = SPLIT || std::is_same<DT, double>::value;
 #pragma unroll
-  for (int j = 0; j < kNPn; ++j) {
+  for (int j = 0; j < kNPn; ++j)
     if (kAllF64 || is_large_pn(j)) sc.alpha[j] = vdbl(alpha[j].v);
-    if (GRAD)
-#pragma unroll
-      for (int i = 0; i < 4; ++i) ec.dalpha[j][i] = alpha[j].d[i];
-  }
   sc.c0 = vdbl(cpn.v) - ph[SHARPY_PHIC] * (1.0 / kTwoPi) - 0.125;
-  if (GRAD)
-#pragma unroll
-    for (int i = 0; i < 4; ++i) ec.dc0[i] = cpn.d[i];
   sc.kisco = isco_bin(ev, fisco);
   if (SPLIT) {
 #pragma unroll
@@ -514,6 +526,17 @@ __device__ void prologue_sky(const DevModel& m, const DevEvent& ev, const double
     for (int a = a0; a < a1; ++a) split2(sc.tau[a], &sc.thi[a], &sc.tlo[a]);
 }
 
+// Sky of detector a. The loop's end is hidden from the compiler: a loop known
+// to run once is contracted into other FMAs than the all-detector loop, a last
+// bit apart.
+template <class DT, bool GRAD, bool SPLIT = false>
+__device__ __forceinline__ void prologue_sky_one(const DevModel& m, const DevEvent& ev, const double* th, int a,
+                                                 SweepCoef& sc, EpiCoef<DT>& ec) {
+  int a1 = a + 1;
+  asm volatile("" : "+r"(a1));
+  prologue_sky<DT, GRAD, SPLIT>(m, ev, th, a, a1, sc, ec);
+}
+
 // theta (free dims) -> sweep and epilogue coefficients.
 template <class DT, bool GRAD, bool SPLIT = false>
 __device__ void prologue(const DevModel& m, const DevEvent& ev, const double* th, SweepCoef& sc,
@@ -533,8 +556,30 @@ __device__ void prologue(const DevModel& m, const DevEvent& ev, const double* th
 template <class DT, bool GRAD, bool SPLIT, class Pos>
 __device__ __forceinline__ void prologue_cta(int warp, int lane, int n, const DevModel& m, const DevEvent& ev,
                                              Pos&& pos, SweepCoef* sc, EpiCoef<DT>* ec) {
-  if (lane >= n || warp >= 2 + ev.n_det) return;
   double th[kMaxDim];
+  if constexpr (std::is_same<DT, double>::value) {
+    // FP64, at most 8 particles: an instruction takes 60 cycles however many
+    // lanes are on, so the lanes of a particle share the phase's directions and
+    // the detectors
+    const int p = lane >> 2, i = lane & 3;
+    if (warp > 2 || p >= n || (warp == 1 && i > 0) || (warp == 2 && i >= ev.n_det)) return;
+    const bool on = pos(p, th);
+    if (warp == 0) {
+      if (on) {
+        prologue_phase<DT, GRAD, false, 1>(m, ev, th, sc[p], ec[p], i);
+      } else if (i == 0) {
+        sc[p].ok = 0;
+        sc[p].kisco = -1;
+      }
+    } else if (on) {
+      if (warp == 1)
+        prologue_amp<DT, GRAD>(m, th, ec[p]);
+      else
+        prologue_sky_one<DT, GRAD>(m, ev, th, i, sc[p], ec[p]);
+    }
+    return;
+  }
+  if (lane >= n || warp >= 2 + ev.n_det) return;
   const bool on = pos(lane, th);
   if (warp == 0) {
     if (on) {
@@ -547,11 +592,7 @@ __device__ __forceinline__ void prologue_cta(int warp, int lane, int n, const De
     if (warp == 1) {
       prologue_amp<DT, GRAD>(m, th, ec[lane]);
     } else {
-      // the end hidden from the compiler: a loop known to run once is contracted
-      // into other FMAs than the all-detector loop, a last bit apart
-      int a1 = warp - 1;
-      asm volatile("" : "+r"(a1));
-      prologue_sky<DT, GRAD, SPLIT>(m, ev, th, warp - 2, a1, sc[lane], ec[lane]);
+      prologue_sky_one<DT, GRAD, SPLIT>(m, ev, th, warp - 2, sc[lane], ec[lane]);
     }
   }
 }
@@ -628,6 +669,94 @@ __device__ void epilogue(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<
   if (GRAD)
 #pragma unroll
     for (int i = 0; i < SHARPY_NPHYS; ++i) gph[i] = (GT)g[i];
+}
+
+// The FP64 path's epilogue on the lanes of one particle: lane (a, p) forms what
+// detector a adds to ln L, to the gradient along mass or spin p and along the
+// p-th of (cos i, psi, ra, sin dec), and to what both share; sums over the
+// detectors follow in their order, so the result does not depend on the number of
+// lanes. About 60 FP64 instructions (60 cycles each, whatever the lanes) where
+// one lane takes 540. Every operation is rounded explicitly: the likelihood and
+// the NUTS kernel, which inline it differently, get the same bits.
+struct EpiPart {
+  double l, gm, gs, gdl, gtc, gph;
+};
+template <bool GRAD>
+__device__ __forceinline__ EpiPart epilogue_part(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<double>& ec,
+                                                 const double* mom, int a, int p) {
+  EpiPart o;
+  const double* M = mom + a * kNMom * 2;
+  const double P = sc.kisco >= 0 ? ev.pref[(int64_t)a * ev.n_bins + sc.kisco] : 0.0;
+  const double a0 = ec.a0, cr = ec.cre[a], ci = ec.cim[a];
+  // Re(C A0 Z) - |C|^2 A0^2 P / 2
+  const double Gr = __dmul_rn(a0, cr), Gi = __dmul_rn(a0, ci);
+  const double G2 = __fma_rn(Gr, Gr, __dmul_rn(Gi, Gi));
+  o.l = __fma_rn(__dmul_rn(-0.5, G2), P, __fma_rn(Gr, M[18], -__dmul_rn(Gi, M[19])));
+  o.gm = o.gs = o.gdl = o.gtc = o.gph = 0.0;
+  if (!GRAD) return o;
+  const double ps = __dmul_rn(ec.A0sq, P), zr = __dmul_rn(a0, M[18]), zi = __dmul_rn(a0, M[19]);
+  // Im(C X) for a scaled phase-derivative moment X
+  auto imcx = [&](double xr, double xi) { return __fma_rn(cr, xi, __dmul_rn(ci, xr)); };
+  double xr = __dmul_rn(ec.dc0[p], M[18]), xi = __dmul_rn(ec.dc0[p], M[19]);
+#pragma unroll
+  for (int j = 0; j < kNPn; ++j) {
+    xr = __fma_rn(ec.dalpha[j][p], M[2 * j], xr);
+    xi = __fma_rn(ec.dalpha[j][p], M[2 * j + 1], xi);
+  }
+  const double ta = __dmul_rn(kTwoPi, a0);
+  o.gm = __dmul_rn(ta, imcx(xr, xi));
+  // Re(dC A0 Z) - Re(conj(C) dC) A0^2 P for a response derivative dC
+  const double dr = ec.dcre[a][p], di = ec.dcim[a][p];
+  o.gs = __fma_rn(-__fma_rn(cr, dr, __dmul_rn(ci, di)), ps, __fma_rn(dr, zr, -__dmul_rn(di, zi)));
+  const double tf = __dmul_rn(ta, imcx(M[16], M[17]));  // per unit of delay
+  if (p >= 2) o.gs = __fma_rn(ec.dtau[a][p - 2], tf, o.gs);
+  const double amp = __fma_rn(-__fma_rn(cr, cr, __dmul_rn(ci, ci)), ps, __fma_rn(cr, zr, -__dmul_rn(ci, zi)));  // d/d ln A0
+  if (p == 0) o.gm = __fma_rn(ec.rel_mc, amp, o.gm);
+  o.gdl = __dmul_rn(ec.rel_dl, amp);
+  o.gtc = tf;
+  o.gph = -imcx(zr, zi);
+  return o;
+}
+
+// Called by a group of G (4, 8 or 16) lanes of mask gm, t = lane in the group;
+// gph: SHARPY_NPHYS values, written for the group (a barrier before they are
+// read is the caller's).
+template <bool GRAD, int G>
+__device__ __forceinline__ void epilogue_lanes(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<double>& ec,
+                                               const double* mom, int t, unsigned gm, double* lnl, double* gph) {
+  constexpr int A = G / 4, ROUNDS = (3 + A - 1) / A;  // detectors at a time
+  const int p = t & 3;
+  EpiPart c[ROUNDS];
+#pragma unroll
+  for (int r = 0; r < ROUNDS; ++r) {
+    const int a = r * A + t / 4;
+    c[r] = a < ev.n_det ? epilogue_part<GRAD>(ev, sc, ec, mom, a, p) : EpiPart{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  }
+  double l = __dmul_rn(-0.5, ev.dd);
+  EpiPart s = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const EpiPart& x = c[a / A];
+    const int from = (a % A) * 4 + p;
+    const double v[6] = {__shfl_sync(gm, x.l, from, G),
+                         GRAD ? __shfl_sync(gm, x.gm, from, G) : 0.0,  GRAD ? __shfl_sync(gm, x.gs, from, G) : 0.0,
+                         GRAD ? __shfl_sync(gm, x.gdl, from, G) : 0.0, GRAD ? __shfl_sync(gm, x.gtc, from, G) : 0.0,
+                         GRAD ? __shfl_sync(gm, x.gph, from, G) : 0.0};
+    if (a >= ev.n_det) continue;
+    l = __dadd_rn(l, v[0]);
+    if (!GRAD) continue;
+    s.gm = __dadd_rn(s.gm, v[1]);
+    s.gs = __dadd_rn(s.gs, v[2]);
+    s.gdl = __dadd_rn(s.gdl, v[3]);
+    s.gtc = __dadd_rn(s.gtc, v[4]);
+    s.gph = __dadd_rn(s.gph, v[5]);
+  }
+  *lnl = l;
+  if (!GRAD || t >= 4) return;
+  static_assert(SHARPY_MC == 0 && SHARPY_CHI2 == 3, "masses and spins first");
+  gph[p] = s.gm;
+  gph[p == 0 ? SHARPY_COSI : p == 1 ? SHARPY_PSI : p == 2 ? SHARPY_RA : SHARPY_SINDEC] = s.gs;
+  if (p < 3) gph[p == 0 ? SHARPY_DL : p == 1 ? SHARPY_TC : SHARPY_PHIC] = p == 0 ? s.gdl : p == 1 ? s.gtc : s.gph;
 }
 
 // Diagonal Gaussian mixture (test targets): ln L and its gradient.
