@@ -11,7 +11,7 @@
 // before (4.8e-13: the phase's rounding).
 //
 // Numbers are 64-bit integers v = h 2^32 + l with both limbs signed; the high
-// word of a product is ah bh + (ah bl + al bh) / 2^32, rounded: 4 multiply-adds,
+// word of a product is ah bh + (ah bl + al bh) / 2^32, rounded: 3 multiply-adds,
 // error under one unit. Errors against the FP64 sweep's, per bin:
 //   phase   the same FP64 sum, then its fraction of a turn exact to 2^-64;
 //   carrier within 2^-58 (a table of 1024 points to 2^-62, sine and cosine of
@@ -54,7 +54,17 @@ struct FixBlock {
 struct Limbs {
   int h, l;
 };
-__host__ __device__ __forceinline__ int64_t fix_mad(int a, int b, int64_t c) { return c + (int64_t)a * b; }
+// c + a b, one instruction: from the plain expression the compiler makes a
+// product and a 64-bit addition (4.3 against 6.7 cycles)
+__host__ __device__ __forceinline__ int64_t fix_mad(int a, int b, int64_t c) {
+#ifdef __CUDA_ARCH__
+  int64_t r;
+  asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+  return r;
+#else
+  return c + (int64_t)a * b;
+#endif
+}
 __host__ __device__ __forceinline__ int fix_hi(int64_t x) { return (int)((uint64_t)x >> 32); }
 __host__ __device__ __forceinline__ Limbs fix_limbs(int64_t v) {
   const uint32_t l = (uint32_t)(uint64_t)v;
@@ -70,7 +80,7 @@ constexpr int64_t kFixHalf = 1LL << 31;
 // c + (a b) / 2^64, rounded; |a b| < 2^125
 __host__ __device__ __forceinline__ int64_t fix_mulhi(Limbs a, Limbs b) {
   const int64_t x = fix_mad(a.l, b.h, fix_mad(a.h, b.l, kFixHalf));
-  return fix_mad(fix_hi(x), 1, fix_mad(a.h, b.h, 0));
+  return fix_mad(a.h, b.h, fix_hi(x));
 }
 __host__ __device__ __forceinline__ uint32_t fix_umulhi(uint32_t a, uint32_t b) {
   return (uint32_t)(((uint64_t)a * b) >> 32);
@@ -135,10 +145,10 @@ constexpr uint32_t kFixB1 = (uint32_t)(147573952589676412928.0 * kFixKappa * kFi
 __host__ __device__ __forceinline__ void fix_small(int64_t rest, int64_t* s, int64_t* c1) {
   const Limbs v = fix_limbs(rest);
   const int64_t x = fix_mad(v.h, v.l, kFixHalf);
-  const int64_t y2 = fix_mad(fix_hi(x), 2, fix_mad(v.h, v.h, 0));  // y^2 2^60, never negative
+  const int64_t y2 = fix_mad(v.h, v.h, 2 * (int64_t)fix_hi(x));  // y^2 2^60, never negative
   const uint32_t Y = (uint32_t)((uint64_t)y2 >> 29);               // y^2 2^31
   const uint32_t t = fix_umulhi(Y, kFixA1 - fix_umulhi(Y, kFixA2));
-  *s = fix_mulhi(v, fix_limbs(fix_mad((int)t, -256, kFixG0)));
+  *s = fix_mulhi(v, fix_limbs(kFixG0 - ((int64_t)t << 8)));
   *c1 = fix_mulhi(fix_limbs(y2), fix_limbs((int64_t)fix_umulhi(Y, kFixB1) - kFixH0));
 }
 
@@ -150,21 +160,30 @@ __host__ __device__ __forceinline__ void fix_carrier(uint64_t u, int4 E, int4 T,
   const Limbs s = fix_limbs_neg(s64), c = fix_limbs(c64);
   // w = E (C - i S) / 4
   int64_t x = fix_mad(E.w, T.z, fix_mad(E.z, T.w, fix_mad(E.y, T.x, fix_mad(E.x, T.y, kFixHalf))));
-  const int64_t wr = fix_mad(fix_hi(x), 1, fix_mad(E.z, T.z, fix_mad(E.x, T.x, 0)));
+  const int64_t wr = fix_mad(E.z, T.z, fix_mad(E.x, T.x, fix_hi(x)));
   x = fix_mad(-E.y, T.z, fix_mad(-E.x, T.w, fix_mad(E.w, T.x, fix_mad(E.z, T.y, kFixHalf))));
-  const int64_t wi = fix_mad(fix_hi(x), 1, fix_mad(-E.x, T.z, fix_mad(E.z, T.x, 0)));
+  const int64_t wi = fix_mad(-E.x, T.z, fix_mad(E.z, T.x, fix_hi(x)));
   // z = w (cos d - i sin d)
   const Limbs r = fix_limbs(wr), i = fix_limbs(wi);
   x = fix_mad(i.l, s.h, fix_mad(i.h, s.l, fix_mad(r.l, c.h, fix_mad(r.h, c.l, kFixHalf))));
-  *zr = fix_mad(fix_hi(x), 1, fix_mad(i.h, s.h, fix_mad(r.h, c.h, wr)));
+  *zr = fix_mad(i.h, s.h, fix_mad(r.h, c.h, wr + fix_hi(x)));
   x = fix_mad(r.l, -s.h, fix_mad(r.h, -s.l, fix_mad(i.l, c.h, fix_mad(i.h, c.l, kFixHalf))));
-  *zi = fix_mad(fix_hi(x), 1, fix_mad(r.h, -s.h, fix_mad(i.h, c.h, wi)));
+  *zi = fix_mad(r.h, -s.h, fix_mad(i.h, c.h, wi + fix_hi(x)));
 }
 
-// acc + (z B) / 2^64, rounded
+// acc + (z B) / 2^64, rounded, + 2^31: the offset makes the cross products' high
+// word unsigned, which saves its sign extension (14 against 16.5 cycles a
+// moment); a sum of n terms starts at fix_start(n).
+constexpr uint64_t kFixBias = 1ULL << 63;
+__host__ __device__ __forceinline__ int64_t fix_start(int n) { return -((int64_t)n << 31); }
 __host__ __device__ __forceinline__ int64_t fix_moment(Limbs z, int bh, int bl, int64_t acc) {
-  const int64_t x = fix_mad(z.l, bh, fix_mad(z.h, bl, kFixHalf));
-  return fix_mad(fix_hi(x), 1, fix_mad(z.h, bh, acc));
+  const int64_t x = fix_mad(z.l, bh, fix_mad(z.h, bl, (int64_t)(kFixBias + (uint64_t)kFixHalf)));
+  return acc + fix_mad(z.h, bh, (int64_t)((uint64_t)x >> 32));
+}
+// the same for a basis value of a high limb alone
+__host__ __device__ __forceinline__ int64_t fix_moment1(Limbs z, int bh, int64_t acc) {
+  const int64_t x = fix_mad(z.l, bh, (int64_t)(kFixBias + (uint64_t)kFixHalf));
+  return acc + fix_mad(z.h, bh, (int64_t)((uint64_t)x >> 32));
 }
 
 }  // namespace sharpy

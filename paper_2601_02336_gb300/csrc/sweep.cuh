@@ -506,14 +506,15 @@ __device__ bool fixed_stream(const DevEvent& ev, const SweepCoef& sc, int s, dou
   for (int g = s * kPer; g * kFixBins <= kend; g += (g % kPer == kPer - 1 ? (kStreams - 1) * kPer : 0) + 1) {
     any = true;
     int64_t acc[NACC];
+    const int kstop = min(kend, g * kFixBins + kFixBins - 1), k0 = g * kFixBins + lane;
+    const int64_t start = fix_start(k0 <= kstop ? (kstop - k0) / 32 + 1 : 0);
 #pragma unroll
-    for (int i = 0; i < NACC; ++i) acc[i] = 0;
+    for (int i = 0; i < NACC; ++i) acc[i] = start;
     const FixBlock* fb = ev.fix_block + g;
     const int one = __ldg(&fb->one);
-    const int kstop = min(kend, g * kFixBins + kFixBins - 1);
     const int4* at = ev.tile_fix + (int64_t)g * (kFixBins * kFixQuads) + lane;
 #pragma unroll 1
-    for (int k = g * kFixBins + lane; k <= kstop; k += 32, at += kFixQuads * kTileBins) {
+    for (int k = k0; k <= kstop; k += 32, at += kFixQuads * kTileBins) {
       double S = sc.c0, f = 0.0;
       int bh[kNBasis], bl[kNBasis];
 #pragma unroll
@@ -544,8 +545,8 @@ __device__ bool fixed_stream(const DevEvent& ev, const SweepCoef& sc, int s, dou
           }
         }
         int64_t* m = acc + (GRAD ? (a * kNMom + 9) * 2 : a * 2);
-        m[0] = fix_moment(r, one, 0, m[0]);
-        m[1] = fix_moment(i, one, 0, m[1]);
+        m[0] = fix_moment1(r, one, m[0]);
+        m[1] = fix_moment1(i, one, m[1]);
       }
     }
     int64_t v[F::NP];
