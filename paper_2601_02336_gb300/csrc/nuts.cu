@@ -69,13 +69,16 @@ int enqueue_nuts(sharpy_ctx* c, int64_t n, const double* beta_ptr, double beta, 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // FP64: 16 slots once they give about 1.5 CTAs an SM. Mixed paths: 8 slots
+    // FP64 (two CTAs of four warps an SM, sweeps much longer than the rest of a
+    // tick): 4 slots while they fit one wave, then 8 (1001 particles 3.89 ms with
+    // 4 slots, 4.45 with 8; 2048: 7.83 and 5.41; 5000: 14.9 with 8, 18.3 with 16).
+    // Mixed paths: 8 slots
     // while one CTA an SM holds them (2048 particles: 3.03 ms with 8, 2.86 with
     // 16; 700: 2.29 and 2.78), 16 while they fit one wave (three CTAs of four
     // warps an SM; 5000: 5.19 ms, 5.88 with 32), then 32 (16384: 11.6 ms, 14.2
     // with 16).
     if (precision == SHARPY_FP64)
-      slots = n >= (int64_t)16 * 2 * sms * 3 / 4 ? 16 : 8;
+      slots = n <= (int64_t)4 * 2 * sms ? 4 : 8;
     else
       slots = n <= (int64_t)8 * sms ? 8 : n <= (int64_t)16 * 3 * sms ? 16 : 32;
   }
