@@ -195,6 +195,7 @@ static const int4* fix_trig_host() {
 static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
   DevEvent& ev = c->ev;
   ev.tile_fix = nullptr;
+  ev.fix_bad = nullptr;
   ev.fix_block = nullptr;
   ev.fix_trig = nullptr;
   if (ev.n_bins > kFixMaxBins || ev.n_det > kFixDet) return cudaSuccess;
@@ -215,11 +216,10 @@ static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
   if (e != cudaSuccess) return e;
   fix_scale_kernel<<<(unsigned)blocks, kFixScaleThreads>>>(ev, fc, bad);
   fix_tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, fc, bad, c->d_fix);
-  int b = 1;
   e = cudaGetLastError();
-  if (e == cudaSuccess) e = cudaMemcpy(&b, bad, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess || b) return e;
+  if (e != cudaSuccess) return e;
   ev.tile_fix = c->d_fix;
+  ev.fix_bad = bad;
   ev.fix_block = fc;
   ev.fix_trig = c->d_fix + tiles;
   return cudaSuccess;

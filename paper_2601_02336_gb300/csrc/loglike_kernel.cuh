@@ -1,7 +1,7 @@
 // The standalone likelihood kernel (sharpy_loglike_grad): one CTA of ll_warps
-// warps; warps 0 to 4 compute the particles' prologues (prologue_cta: lane s =
-// particle s of the CTA), the warps sweep the particles' bins, and warp 0
-// finishes with the lane-parallel epilogue. The instantiations of each
+// warps; the first of them compute the particles' prologues (prologue_cta), the
+// warps sweep the particles' bins, and warp 0 finishes with the lane-parallel
+// epilogue (on the FP64 path each particle's first warp, epilogue_lanes). The instantiations of each
 // precision are compiled in their own unit (loglike_inst.cu).
 #pragma once
 #include "bulk.cuh"
@@ -338,7 +338,7 @@ inline cudaError_t launch_ll_split(sharpy_ctx* c, int split, int64_t n, const do
     if constexpr (PREC == SHARPY_MIXED_SPLIT) {
       if (c->ev.n_bins >= kStageMinBins) return launch_ll_staged_split_unit(c, GRAD, NDET, n, th, lnl, grad, s);
     }
-    split = 8;  // no staged tables, or the FP64 path: the 8-warp split
+    split = 8;  // no staged tables, or the FP64 path: all warps of a CTA
   }
   switch (split) {
     case 2: launch_ll_one<PREC, GRAD, NDET, 2>(c, n, th, lnl, grad, s); break;

@@ -634,7 +634,7 @@ __device__ bool fp64_stream(const DevEvent& ev, const SweepCoef& sc, int s, doub
 // One stream of the FP64 path, in the arithmetic that the event's data allow.
 template <bool GRAD, int NDET>
 __device__ bool wide_stream(const DevEvent& ev, const SweepCoef& sc, int s, double* v_out) {
-  return ev.tile_fix ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
+  return ev.tile_fix && *ev.fix_bad == 0 ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
 }
 
 // FP64 moments of one particle on one warp; streams as in sweep_mixed (a
