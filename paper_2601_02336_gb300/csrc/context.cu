@@ -174,13 +174,16 @@ __global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const
 static const int4* fix_trig_host() {
   static const std::vector<int4> t = [] {
     std::vector<int4> v(kFixTrig);
-    const long double w = 6.283185307179586476925286766559L / kFixTrig;
+    constexpr int O = kFixTrig / 8;
+    int64_t co[O + 1], si[O + 1];
+    for (int i = 0; i <= O; ++i) {
+      const long double x = 6.283185307179586476925286766559L / kFixTrig * i;
+      co[i] = (int64_t)std::rint(std::ldexp(std::cos(x), 62));
+      si[i] = (int64_t)std::rint(std::ldexp(std::sin(x), 62));
+    }
     for (int i = 0; i < kFixTrig; ++i) {
-      const int q = i * 4 / kFixTrig, r = i % (kFixTrig / 4);  // quadrant, place in it
-      const bool swap = r > kFixTrig / 8;
-      const long double x = w * (swap ? kFixTrig / 4 - r : r);
-      const int64_t a = (int64_t)std::rint(std::ldexp(swap ? std::sin(x) : std::cos(x), 62));
-      const int64_t b = (int64_t)std::rint(std::ldexp(swap ? std::cos(x) : std::sin(x), 62));
+      const int q = i / (2 * O), r = i % (2 * O);  // quadrant, place in it
+      const int64_t a = r > O ? si[2 * O - r] : co[r], b = r > O ? co[2 * O - r] : si[r];
       const Limbs c = fix_limbs_neg(q == 0 ? a : q == 1 ? -b : q == 2 ? -a : b);
       const Limbs s = fix_limbs_neg(q == 0 ? b : q == 1 ? a : q == 2 ? -b : -a);
       v[i] = make_int4(c.h, c.l, s.h, s.l);
