@@ -93,7 +93,7 @@ struct DevEvent {
   const float4* tile_mixed;  // tiles of the mixed and the split sweep, whole blocks of kStageBins
   const float4* tile_split;
   const int4* tile_fix;      // the FP64 path's bins in fixed point (fixed.cuh), or null: the FP64 sweep
-  const int* fix_bad;        // nonzero: the staged data take the FP64 sweep (read by the kernels: it goes with the tables)
+  const int* fix_from;       // sweeps whose last active bin lies below take the FP64 sweep (read by the kernels: it goes with the tables)
   const FixBlock* fix_block; // their scales, per block of 256 bins
   const int4* fix_trig;      // the carrier's table
   const double* pref;        // [n_det][K] prefix sums of w f^-7/3

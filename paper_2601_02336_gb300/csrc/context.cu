@@ -72,85 +72,136 @@ __global__ void __launch_bounds__(kStageBins) tile_kernel(DevEvent ev, float4* m
 // Scales of one block of 256 bins per CTA. E_a takes 2^e with 2^e |E| <= 2^61; basis
 // function j the largest 2^b with 2^b |B| <= 2^61 for which no sum of the
 // block's products can reach 2^62 (the integer sums' high words; z is in E's
-// units / 4); the basis value 1 likewise. *bad: data that no
-// scale fits, or whose first tile lies below 2^-6 of its largest value.
+// units / 4); the basis value 1 likewise. *from: past the tiles of block 0 in
+// which a sweep must not end (fix_fails), or kFixNever for data that no scale
+// fits (largest values outside 2^-200 .. 2^200, where FP64 holds the squares).
 constexpr int kFixScaleThreads = 1024;
 static_assert(kFixDet * kNMom * 32 <= kFixScaleThreads, "a warp a moment");
 static_assert(kFixBins == kStageBins, "the tiles' blocks");
-__global__ void __launch_bounds__(kFixScaleThreads) fix_scale_kernel(DevEvent ev, FixBlock* out, int* bad) {
-  __shared__ double emax[2][kFixDet], bmax[2][kNBasis], sum[kFixDet][kNMom];  // [0]: first tile, [1]: block
+__global__ void __launch_bounds__(kFixScaleThreads) fix_scale_kernel(DevEvent ev, FixBlock* out, FixGuard* guard, int* from) {
+  constexpr int T = kFixBins / kTileBins;
+  __shared__ double emax[kFixDet], bmax[kNBasis], sum[kFixDet][kNMom];
+  __shared__ int fits;
   const int64_t K = ev.n_bins, k0 = (int64_t)blockIdx.x * kFixBins;
-  const int64_t k1 = k0 + kFixBins < K ? k0 + kFixBins : K;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // warp w: moment (a, j) = (w / 10, w % 10) of up to 30
   const int a = warp / kNMom, j = warp % kNMom;
   const bool on = a < ev.n_det;
-  double em = 0.0, bm = 0.0, s = 0.0, em0 = 0.0, bm0 = 0.0;
+  double em = 0.0, bm = 0.0, s = 0.0, q[T];  // q[t]: squares of tile t
   bool fin = true;
-  if (on)
-    for (int64_t k = k0 + lane; k < k1; k += 32) {
-      const double2 e = ev.e64[a * K + k];
-      const double b = j < kNBasis ? fabs(ev.b64[j * K + k]) : 1.0;
-      const double l2 = hypot(e.x, e.y), lm = fmax(fabs(e.x), fabs(e.y));
-      fin = fin && isfinite(l2) && isfinite(b);
-      em = fmax(em, lm);
-      bm = fmax(bm, b);
-      if (k < k0 + 32) em0 = lm, bm0 = b;
-      s = fma(l2, b, s);
-    }
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    const int64_t k = k0 + t * kTileBins + lane;
+    q[t] = 0.0;
+    if (!on || k >= K) continue;
+    const double2 e = ev.e64[a * K + k];
+    const double b = j < kNBasis ? fabs(ev.b64[j * K + k]) : 1.0;
+    const double l2 = hypot(e.x, e.y);
+    fin = fin && isfinite(l2) && isfinite(b);
+    em = fmax(em, fmax(fabs(e.x), fabs(e.y)));
+    bm = fmax(bm, b);
+    s = fma(l2, b, s);
+    q[t] = l2 * b * (l2 * b);
+  }
 #pragma unroll
   for (int o = 16; o >= 1; o >>= 1) {
     em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
     bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-    em0 = fmax(em0, __shfl_xor_sync(0xffffffffu, em0, o));
-    bm0 = fmax(bm0, __shfl_xor_sync(0xffffffffu, bm0, o));
     s += __shfl_xor_sync(0xffffffffu, s, o);
+#pragma unroll
+    for (int t = 0; t < T; ++t) q[t] += __shfl_xor_sync(0xffffffffu, q[t], o);
   }
   fin = __all_sync(0xffffffffu, fin);
+  if (threadIdx.x == 0) fits = 1;
+  __syncthreads();
   if (on && lane == 0) {
-    if (!fin || !isfinite(s)) atomicExch(bad, 1);
+    if (!fin || !isfinite(s)) fits = 0;
     sum[a][j] = s;
-    if (j == 0) emax[0][a] = em0, emax[1][a] = em;
-    if (a == 0 && j < kNBasis) bmax[0][j] = bm0, bmax[1][j] = bm;
+    if (j == 0) emax[a] = em;
+    if (a == 0 && j < kNBasis) bmax[j] = bm;
   }
   __syncthreads();
-  if (threadIdx.x != 0) return;
   FixBlock& fc = out[blockIdx.x];
-  int ee[kFixDet];
-  bool ok = true;
-  for (int i = 0; i < ev.n_det; ++i) {
-    const double m = emax[1][i];
-    ok = ok && (m == 0.0 || (isfinite(m) && m >= 1e-250 && emax[0][i] >= m * 0.015625));
-    ee[i] = m > 0.0 && ok ? 60 - ilogb(m) : 0;
-  }
-  for (int n = 0; n < kNMom; ++n) {
-    int be = 29 + 32;  // the basis value 1, a high limb alone
-    if (n < kNBasis) {
-      const double m = bmax[1][n];
-      ok = ok && (m == 0.0 || (isfinite(m) && m >= 1e-250 && bmax[0][n] >= m * 0.015625));
-      be = m > 0.0 && ok ? 60 - ilogb(m) : 0;
-    }
-    for (int i = 0; i < ev.n_det; ++i)
-      if (ok && sum[i][n] > 0.0) be = min(be, 127 - ee[i] - ilogb(sum[i][n]));
-    if (n == kNBasis) {
-      ok = ok && be >= 32;
-      fc.one = ok ? 1 << (be - 32) : 0;
-    }
+  if (threadIdx.x == 0) {
+    int ee[kFixDet];
+    bool ok = fits != 0;
+    auto fit = [&](double m) { return m == 0.0 || (m >= 0x1p-200 && m <= 0x1p200); };
     for (int i = 0; i < ev.n_det; ++i) {
-      ok = ok && abs(66 - ee[i] - be) <= 1000;
-      fc.scale[i * kNMom + n] = ldexp(1.0, ok ? 66 - ee[i] - be : 0);
+      ok = ok && fit(emax[i]);
+      ee[i] = emax[i] > 0.0 && ok ? 60 - ilogb(emax[i]) : 0;
     }
-    fc.be[n] = be;
+    for (int n = 0; n < kNMom; ++n) {
+      int be = 29 + 32;  // the basis value 1, a high limb alone
+      if (n < kNBasis) {
+        ok = ok && fit(bmax[n]);
+        be = bmax[n] > 0.0 && ok ? 60 - ilogb(bmax[n]) : 0;
+      }
+      for (int i = 0; i < ev.n_det; ++i)
+        if (ok && sum[i][n] > 0.0) be = min(be, 127 - ee[i] - ilogb(sum[i][n]));
+      if (n == kNBasis) {
+        ok = ok && be >= 32;
+        fc.one = ok ? 1 << (be - 32) : 0;
+      }
+      for (int i = 0; i < ev.n_det; ++i) {
+        ok = ok && abs(66 - ee[i] - be) <= 1000;
+        fc.scale[i * kNMom + n] = ldexp(1.0, ok ? 66 - ee[i] - be : 0);
+      }
+      fc.be[n] = be;
+    }
+    for (int i = 0; i < ev.n_det; ++i) fc.ee[i] = ee[i];
+    fits = ok;
+    if (!ok) atomicMax(from, kFixNever);
   }
-  for (int i = 0; i < ev.n_det; ++i) fc.ee[i] = ee[i];
-  if (!ok) atomicExch(bad, 1);
+  __syncthreads();
+  if (!on || lane != 0) return;
+  const int n = a * kNMom + j;
+  const double unit = fc.scale[n];
+  double sq = 0.0, need = 0.0;
+  int last = 0;  // block 0: the last tile in which an end fails
+  // (products that are all zero are exact)
+#pragma unroll
+  for (int t = 0; t < T; ++t) {
+    if (s > 0.0 && fix_fails(unit, t, sq)) {
+      need = fmax(need, fix_need(unit, t) - sq);
+      last = t;
+    }
+    sq += q[t];
+  }
+  guard[blockIdx.x].sq[n] = sq;
+  guard[blockIdx.x].need[n] = blockIdx.x == 0 ? 0.0 : need;
+  if (blockIdx.x == 0) atomicMax(from, kTileBins * (last + 1));
+}
+
+// fix_from over all blocks: one CTA, a warp a moment, lanes over the blocks; an
+// exclusive prefix sum of the blocks' squares against what each needs before
+// it. *from rises past the last block that fails.
+__global__ void __launch_bounds__(kFixScaleThreads) fix_guard_kernel(int n_det, int64_t blocks, const FixGuard* guard, int* from) {
+  const int n = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (n >= n_det * kNMom) return;
+  double before = 0.0;
+  int last = -1;
+  for (int64_t g0 = 0; g0 < blocks; g0 += 32) {
+    const int64_t g = g0 + lane;
+    const double sq = g < blocks ? guard[g].sq[n] : 0.0;
+    double incl = sq;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    double excl = __shfl_up_sync(0xffffffffu, incl, 1);
+    excl = before + (lane ? excl : 0.0);
+    if (g < blocks && !(guard[g].need[n] <= excl)) last = (int)g;
+    before += __shfl_sync(0xffffffffu, incl, 31);
+  }
+  if (last >= 0) atomicMax(from, (last + 1) * kFixBins);
 }
 
 // One CTA per block of kStageBins bins, one thread per bin: the bin's
 // fixed-point quads (zeros past the last bin).
-__global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const FixBlock* fc, const int* bad, int4* out) {
-  if (*bad) return;
+__global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const FixBlock* fc, const int* from, int4* out) {
   const int64_t K = ev.n_bins, k = (int64_t)blockIdx.x * kStageBins + threadIdx.x;
+  if (*from >= K) return;
   const bool in = k < K;
   const FixBlock& c = fc[k / kFixBins];
   int4* t = out + k / kTileBins * (kFixQuads * kTileBins) + k % kTileBins;
@@ -198,14 +249,14 @@ static const int4* fix_trig_host() {
 static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
   DevEvent& ev = c->ev;
   ev.tile_fix = nullptr;
-  ev.fix_bad = nullptr;
+  ev.fix_from = nullptr;
   ev.fix_block = nullptr;
   ev.fix_trig = nullptr;
   if (ev.n_bins > kFixMaxBins || ev.n_det > kFixDet) return cudaSuccess;
   const size_t tiles = (size_t)blocks * kStageBins * kFixQuads;
-  const size_t scales = (size_t)((ev.n_bins + kFixBins - 1) / kFixBins);
   if (!c->d_fix) {
-    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig) * sizeof(int4) + (size_t)blocks * sizeof(FixBlock) + sizeof(int)) != cudaSuccess) {
+    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig) * sizeof(int4) + (size_t)blocks * (sizeof(FixBlock) + sizeof(FixGuard)) +
+                                  sizeof(int)) != cudaSuccess) {
       c->d_fix = nullptr;
       (void)cudaGetLastError();
       return cudaSuccess;
@@ -214,15 +265,17 @@ static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
     if (e != cudaSuccess) return e;
   }
   FixBlock* fc = reinterpret_cast<FixBlock*>(c->d_fix + tiles + kFixTrig);
-  int* bad = reinterpret_cast<int*>(fc + blocks);
-  cudaError_t e = cudaMemset(bad, 0, sizeof(int));
+  FixGuard* guard = reinterpret_cast<FixGuard*>(fc + blocks);
+  int* from = reinterpret_cast<int*>(guard + blocks);
+  cudaError_t e = cudaMemset(from, 0, sizeof(int));
   if (e != cudaSuccess) return e;
-  fix_scale_kernel<<<(unsigned)blocks, kFixScaleThreads>>>(ev, fc, bad);
-  fix_tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, fc, bad, c->d_fix);
+  fix_scale_kernel<<<(unsigned)blocks, kFixScaleThreads>>>(ev, fc, guard, from);
+  fix_guard_kernel<<<1, kFixScaleThreads>>>(ev.n_det, blocks, guard, from);
+  fix_tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, fc, from, c->d_fix);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   ev.tile_fix = c->d_fix;
-  ev.fix_bad = bad;
+  ev.fix_from = from;
   ev.fix_block = fc;
   ev.fix_trig = c->d_fix + tiles;
   return cudaSuccess;
@@ -469,6 +522,17 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   ev.tile_mixed = c->d_tile;
   ev.tile_split = split;
   c->has_data = true;
+  return SHARPY_OK;
+}
+
+int sharpy_fixed_point_from(sharpy_ctx* c, int64_t* bin) {
+  int rc = check_ctx(c, true);
+  if (rc) return rc;
+  if (!bin) return SHARPY_EINVAL;
+  if (c->model.model != SHARPY_MODEL_TAYLORF2) return SHARPY_EINVAL;
+  int from = kFixNever;
+  if (c->ev.tile_fix) SHARPY_CUDA_TRY(cudaMemcpy(&from, c->ev.fix_from, sizeof(int), cudaMemcpyDeviceToHost));
+  *bin = from < c->ev.n_bins ? from : c->ev.n_bins;
   return SHARPY_OK;
 }
 

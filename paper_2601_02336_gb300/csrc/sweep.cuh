@@ -9,7 +9,7 @@
 //
 //   SHARPY_FP64  : the phase in FP64; carrier, data product and moments in
 //                  64-bit fixed point (fixed.cuh: errors below FP64's), or, for
-//                  data that it does not fit, FP64 throughout (reduction
+//                  data and ends that it does not fit, FP64 throughout (reduction
 //                  Psi - rint(Psi); sincospi).
 //   SHARPY_MIXED_SPLIT : as SHARPY_MIXED, but the phase polynomial is built
 //                  from hi/lo FP32 splits of alpha_j, tau_a and B_j(f_k):
@@ -631,10 +631,11 @@ __device__ bool fp64_stream(const DevEvent& ev, const SweepCoef& sc, int s, doub
   return any;
 }
 
-// One stream of the FP64 path, in the arithmetic that the event's data allow.
+// One stream of the FP64 path, in the arithmetic that the event's data allow
+// for a sweep of this length (fixed.cuh).
 template <bool GRAD, int NDET>
 __device__ bool wide_stream(const DevEvent& ev, const SweepCoef& sc, int s, double* v_out) {
-  return ev.tile_fix && *ev.fix_bad == 0 ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
+  return ev.tile_fix && sc.kisco >= *ev.fix_from ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
 }
 
 // FP64 moments of one particle on one warp; streams as in sweep_mixed (a

@@ -378,3 +378,71 @@ def test_loglike_fp64_block_edges(name, n_bins, outlier):
         assert np.all(err <= np.maximum(1e-8 * norm, 1e-6)), split
     assert all(torch.equal(a, b) for a, b in zip(*out))
     assert ctx.status() == 0
+
+
+def _cut_at(w, th, bins):
+    """th with masses whose last active bins are `bins`."""
+    out = np.tile(th, (len(bins), 1))
+    q = 0.3
+    for row, k in zip(out, bins):
+        m = 1.0 / (6.0 ** 1.5 * np.pi * 4.925491025543576e-6 * (w.f_min + (k + 0.5) * w.df))
+        row[w.phys.index(inputs.MC)] = m * q ** 0.6 / (1.0 + q) ** 1.2
+        row[w.phys.index(inputs.Q)] = q
+    return out
+
+
+@pytest.mark.parametrize("bin_", [1, 5, 20, 31, 32, 256, 257, 276, 287, 300])
+def test_loglike_fp64_outlier_past_the_end(bin_):
+    """One bin scaled up by 2^0 to 2^40, in the first tile of a block and elsewhere, and vectors that end around it:
+    those that end before the bin must not lose bits to its scale. Within the FP64 path's bounds of the oracle (ln L
+    1e-7 + 1e-10 |ln L|, the gradient 1e-8 of its norm in prior widths, or 1e-6 where the norm is below the ln L
+    bound's scale), each vector as alone, and in the arithmetic that the event's rule gives: without an outlier fixed
+    point from the first tile on, with a large one only past its tile."""
+    G.require_gpu()
+    w = inputs.bbh11()
+    w.f_min, w.n_bins = 40.0, 600
+    _, ctx, th_inj, data0 = G.event_pair(w, seed=0)
+    wid = G.width(w)
+    ends = sorted({max(bin_ - d, 0) for d in (0, 1, 4, 12)} | {bin_ + 3, bin_ + 40, 500})
+    th = _cut_at(w, th_inj, ends)
+    for p in (0, 4, 10, 20, 30, 40):
+        data = data0.copy()
+        data[:, bin_] *= 2.0 ** p
+        ctx.set_data(data, inputs.psd_array(w), w.f_min, w.df, inputs.detectors(w))
+        ref_l, ref_g = oracle.loglike(helpers.oracle_model(w), helpers.oracle_event(w, data=data), th)
+        norm = np.linalg.norm(ref_g * wid, axis=1)
+        l, g = ctx.loglike_grad(G.to_dev(th), "fp64")
+        l0, _ = ctx.loglike_grad(G.to_dev(th), "fp64", grad=False)
+        for x in (l, l0):
+            assert np.all(np.abs(x.cpu().numpy() - ref_l) <= 1e-7 + 1e-10 * np.abs(ref_l)), p
+        err = np.linalg.norm((g.cpu().numpy() - ref_g) * wid, axis=1)
+        assert np.all(err <= np.maximum(1e-8 * norm, 1e-6)), (p, err / norm)
+        for i in range(len(th)):
+            li, gi = ctx.loglike_grad(G.to_dev(th[i:i + 1]), "fp64")
+            assert torch.equal(li[0], l[i]) and torch.equal(gi[0], g[i]), (p, i)
+        at = ctx.fixed_point_from()
+        if p == 0 or bin_ < 32:
+            assert at == 32
+        elif p >= 20:
+            assert at == (bin_ // 32 + 1) * 32 if bin_ < 256 else at == 512
+    assert ctx.status() == 0
+
+
+def test_loglike_fp64_data_without_a_scale():
+    """Data that no scale fits (pre-whitened by a PSD 2^300 times smaller) take the FP64 sweep throughout and give the
+    ordinary ln L and gradient times 2^300; zeros need no scale."""
+    G.require_gpu()
+    w = inputs.tiny()
+    ev, ctx, th_inj, data = G.event_pair(w, seed=0)
+    th = G.to_dev(inputs.ball(w, th_inj, 5, 52))
+    psd = inputs.psd_array(w)
+    l, g = ctx.loglike_grad(th, "fp64")
+    assert ctx.fixed_point_from() == 32
+    ctx.set_data(np.zeros_like(data), psd, w.f_min, w.df, inputs.detectors(w))
+    assert ctx.fixed_point_from() == 32
+    ctx.set_data(data, psd * 2.0 ** -300, w.f_min, w.df, inputs.detectors(w))
+    assert ctx.fixed_point_from() == w.n_bins
+    big, gbig = ctx.loglike_grad(th, "fp64")
+    assert torch.allclose(big * 2.0 ** -300, l, rtol=1e-12, atol=0.0)
+    assert torch.allclose(gbig * 2.0 ** -300, g, rtol=1e-9, atol=1e-9 * float(g.abs().max()))
+    assert ctx.status() == 0
