@@ -30,192 +30,233 @@ int check_ctx(sharpy_ctx* ctx, bool need_data) {
   return SHARPY_OK;
 }
 
-// One CTA per block of kStageBins bins, one thread per bin: writes the bin's
-// quads of the mixed and of the split sweep's tiles.
-__global__ void __launch_bounds__(kStageBins) tile_kernel(DevEvent ev, float4* mixed, float4* split) {
+// Tables of one event, one CTA per block of kStageBins bins, one thread per bin,
+// one warp per tile: the bin's quads of the mixed and of the split sweep's
+// tiles and, if fix.tile is not null, of the FP64 path's in fixed point with the
+// block's scales and what it brings to the rule on the sweeps' ends.
+// Scales: E_a takes 2^e with 2^e |E| <= 2^61; basis function j the largest 2^b
+// with 2^b |B| <= 2^61 for which no sum of the block's products can reach 2^62
+// (the integer sums' high words; z is in E's units / 4); the basis value 1
+// likewise. They come from the largest values' exponents, the products' sums in
+// units of 2^-17 of the two powers of two, rounded up, and their squares in 2^-21,
+// rounded down, so that a warp sums them with one integer instruction each. Bound
+// by latency (32 CTAs for 8033 bins), which the host's own sums hide: a data set
+// on the same grid takes 0.21 ms (433 bins: 0.05), without the fixed-point
+// tables 0.23 (0.03); with a kernel of 30 warps a block, a moment each in FP64,
+// before one for the limbs it took 0.33 (0.11).
+struct FixTables {
+  int4* tile;
+  FixBlock* block;
+  double *sq, *need;   // [kFixDet * kNMom][blocks]
+  int* from;           // [blocks], then the event's fix_from
+  unsigned int* done;  // blocks that have written these; zero between launches
+};
+__device__ __forceinline__ uint32_t fix_abs_hi(double x) {  // |x|'s high word, zero for zero only
+  return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0);
+}
+__device__ __forceinline__ double fix_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// fix_from over all blocks, on the CTA that comes last: a warp a moment in turn,
+// lanes over the blocks; an exclusive prefix sum of the blocks' squares against
+// what each needs before it. Past the last block that fails, or what the blocks
+// ask for themselves.
+__device__ void fix_from_all(int n_det, int blocks, const FixTables& fix) {
+  __shared__ int from_s;
+  const int lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) from_s = 0;
+  __syncthreads();
+  int from = 0;
+  for (int g = threadIdx.x; g < blocks; g += blockDim.x) from = max(from, __ldcg(fix.from + g));
+  for (int n = threadIdx.x >> 5; n < n_det * kNMom; n += blockDim.x >> 5) {
+    const double *sqs = fix.sq + (int64_t)n * blocks, *needs = fix.need + (int64_t)n * blocks;
+    double before = 0.0;
+    for (int g0 = 0; g0 < blocks; g0 += 32) {
+      const int g = g0 + lane;
+      double incl = g < blocks ? __ldcg(sqs + g) : 0.0;
+      const double need = g < blocks ? __ldcg(needs + g) : 0.0;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const double x = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += x;
+      }
+      const double excl = __shfl_up_sync(0xffffffffu, incl, 1);
+      if (!(need <= before + (lane ? excl : 0.0))) from = max(from, (g + 1) * kFixBins);
+      before += __shfl_sync(0xffffffffu, incl, 31);
+    }
+  }
+  atomicMax(&from_s, from);
+  __syncthreads();
+  if (threadIdx.x == 0) fix.from[blocks] = from_s;
+}
+
+static_assert(kFixBins == kStageBins, "one block size");
+__global__ void __launch_bounds__(kStageBins)
+    event_tables_kernel(DevEvent ev, float4* mixed, float4* split, FixTables fix) {
+  constexpr int T = kFixBins / kTileBins, NV = kFixDet + kNBasis, NM = kFixDet * kNMom;
   const int64_t K = ev.n_bins, k = (int64_t)blockIdx.x * kStageBins + threadIdx.x;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const bool in = k < K;
   double b[kNBasis];
-  float hi[kNBasis], lo[kNBasis];
-  float2 E[3];
-  for (int j = 0; j < kNBasis; ++j) {
-    b[j] = in ? ev.b64[j * K + k] : 0.0;
-    hi[j] = (float)b[j];
-    lo[j] = (float)(b[j] - (double)hi[j]);
-  }
-  for (int a = 0; a < 3; ++a) {
-    const double2 e = in && a < ev.n_det ? ev.e64[a * K + k] : make_double2(0.0, 0.0);
-    E[a] = make_float2((float)e.x, (float)e.y);
-  }
-  auto words = [&](bool sp, const float* t, int i) {
-    return make_float4(t[tile_basis(sp, i)], t[tile_basis(sp, i + 1)], t[tile_basis(sp, i + 2)], t[tile_basis(sp, i + 3)]);
-  };
+  double2 e[kFixDet];
+#pragma unroll
+  for (int j = 0; j < kNBasis; ++j) b[j] = in ? ev.b64[j * K + k] : 0.0;
+#pragma unroll
+  for (int a = 0; a < kFixDet; ++a) e[a] = in && a < ev.n_det ? ev.e64[a * K + k] : make_double2(0.0, 0.0);
   const int64_t tile = k / kTileBins;
-  const int lane = (int)(k % kTileBins);
-  float4* m = mixed + tile * tile_quads(false) * kTileBins + lane;
-  m[0 * kTileBins] = words(false, hi, 0);
-  m[1 * kTileBins] = words(false, hi, 4);
-  m[2 * kTileBins] = words(false, lo, 0);
-  m[3 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
-  m[4 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
-  for (int i = 0; i < 2; ++i)
-    reinterpret_cast<double2*>(m)[(5 + i) * kTileBins] = make_double2(b[large_pn(2 * i)], b[large_pn(2 * i + 1)]);
-  float4* s = split + tile * tile_quads(true) * kTileBins + lane;
-  s[0 * kTileBins] = words(true, hi, 0);
-  s[1 * kTileBins] = words(true, hi, 4);
-  s[2 * kTileBins] = words(true, lo, 0);
-  s[3 * kTileBins] = words(true, lo, 4);
-  s[4 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
-  s[5 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
-}
-
-// Scales of one block of 256 bins per CTA. E_a takes 2^e with 2^e |E| <= 2^61; basis
-// function j the largest 2^b with 2^b |B| <= 2^61 for which no sum of the
-// block's products can reach 2^62 (the integer sums' high words; z is in E's
-// units / 4); the basis value 1 likewise. *from: past the tiles of block 0 in
-// which a sweep must not end (fix_fails), or kFixNever for data that no scale
-// fits (largest values outside 2^-200 .. 2^200, where FP64 holds the squares).
-constexpr int kFixScaleThreads = 1024;
-static_assert(kFixDet * kNMom * 32 <= kFixScaleThreads, "a warp a moment");
-static_assert(kFixBins == kStageBins, "the tiles' blocks");
-__global__ void __launch_bounds__(kFixScaleThreads) fix_scale_kernel(DevEvent ev, FixBlock* out, FixGuard* guard, int* from) {
-  constexpr int T = kFixBins / kTileBins;
-  __shared__ double emax[kFixDet], bmax[kNBasis], sum[kFixDet][kNMom];
-  __shared__ int fits;
-  const int64_t K = ev.n_bins, k0 = (int64_t)blockIdx.x * kFixBins;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // warp w: moment (a, j) = (w / 10, w % 10) of up to 30
-  const int a = warp / kNMom, j = warp % kNMom;
-  const bool on = a < ev.n_det;
-  double em = 0.0, bm = 0.0, s = 0.0, q[T];  // q[t]: squares of tile t
-  bool fin = true;
+  {
+    float hi[kNBasis], lo[kNBasis];
+    float2 E[kFixDet];
 #pragma unroll
-  for (int t = 0; t < T; ++t) {
-    const int64_t k = k0 + t * kTileBins + lane;
-    q[t] = 0.0;
-    if (!on || k >= K) continue;
-    const double2 e = ev.e64[a * K + k];
-    const double b = j < kNBasis ? fabs(ev.b64[j * K + k]) : 1.0;
-    const double l2 = hypot(e.x, e.y);
-    fin = fin && isfinite(l2) && isfinite(b);
-    em = fmax(em, fmax(fabs(e.x), fabs(e.y)));
-    bm = fmax(bm, b);
-    s = fma(l2, b, s);
-    q[t] = l2 * b * (l2 * b);
+    for (int j = 0; j < kNBasis; ++j) {
+      hi[j] = (float)b[j];
+      lo[j] = (float)(b[j] - (double)hi[j]);
+    }
+#pragma unroll
+    for (int a = 0; a < kFixDet; ++a) E[a] = make_float2((float)e[a].x, (float)e[a].y);
+    auto words = [&](bool sp, const float* t, int i) {
+      return make_float4(t[tile_basis(sp, i)], t[tile_basis(sp, i + 1)], t[tile_basis(sp, i + 2)], t[tile_basis(sp, i + 3)]);
+    };
+    float4* m = mixed + tile * tile_quads(false) * kTileBins + lane;
+    m[0 * kTileBins] = words(false, hi, 0);
+    m[1 * kTileBins] = words(false, hi, 4);
+    m[2 * kTileBins] = words(false, lo, 0);
+    m[3 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
+    m[4 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
+    for (int i = 0; i < 2; ++i)
+      reinterpret_cast<double2*>(m)[(5 + i) * kTileBins] = make_double2(b[large_pn(2 * i)], b[large_pn(2 * i + 1)]);
+    float4* s = split + tile * tile_quads(true) * kTileBins + lane;
+    s[0 * kTileBins] = words(true, hi, 0);
+    s[1 * kTileBins] = words(true, hi, 4);
+    s[2 * kTileBins] = words(true, lo, 0);
+    s[3 * kTileBins] = words(true, lo, 4);
+    s[4 * kTileBins] = make_float4(hi[8], lo[8], E[0].x, E[0].y);
+    s[5 * kTileBins] = make_float4(E[1].x, E[1].y, E[2].x, E[2].y);
   }
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    em = fmax(em, __shfl_xor_sync(0xffffffffu, em, o));
-    bm = fmax(bm, __shfl_xor_sync(0xffffffffu, bm, o));
-    s += __shfl_xor_sync(0xffffffffu, s, o);
-#pragma unroll
-    for (int t = 0; t < T; ++t) q[t] += __shfl_xor_sync(0xffffffffu, q[t], o);
-  }
-  fin = __all_sync(0xffffffffu, fin);
-  if (threadIdx.x == 0) fits = 1;
+  if (!fix.tile) return;
+  __shared__ uint32_t top[NV], sum_s[T][NM], sq_s[T][NM];
+  __shared__ int be_s[kNBasis], last_s;
+  // the largest values of E_a (either part) and of B_j, as high words
+  if (threadIdx.x < NV) top[threadIdx.x] = 0;
   __syncthreads();
-  if (on && lane == 0) {
-    if (!fin || !isfinite(s)) fits = 0;
-    sum[a][j] = s;
-    if (j == 0) emax[a] = em;
-    if (a == 0 && j < kNBasis) bmax[j] = bm;
+  {
+    uint32_t own = 0;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const uint32_t h = i < kFixDet ? max(fix_abs_hi(e[i < kFixDet ? i : 0].x), fix_abs_hi(e[i < kFixDet ? i : 0].y))
+                                     : fix_abs_hi(b[i < kFixDet ? 0 : i - kFixDet]);
+      const uint32_t m = __reduce_max_sync(0xffffffffu, h);
+      if (lane == i) own = m;
+    }
+    if (lane < NV) atomicMax(&top[lane], own);
   }
   __syncthreads();
-  FixBlock& fc = out[blockIdx.x];
-  if (threadIdx.x == 0) {
-    int ee[kFixDet];
-    bool ok = fits != 0;
-    auto fit = [&](double m) { return m == 0.0 || (m >= 0x1p-200 && m <= 0x1p200); };
-    for (int i = 0; i < ev.n_det; ++i) {
-      ok = ok && fit(emax[i]);
-      ee[i] = emax[i] > 0.0 && ok ? 60 - ilogb(emax[i]) : 0;
+  // exponents (zeros: 0); a block with values outside 2^-200 .. 2^200 (past
+  // which FP64 may not hold the squares), infinities or NaN has no scales
+  bool fits = true;
+  auto expo = [&](int i) {
+    const int x = (int)(top[i] >> 20) - 1023;
+    if (top[i] == 0) return 0;
+    fits = fits && x >= -200 && x < 200;
+    return x;
+  };
+  int ea[kFixDet], eb[kNMom];
+#pragma unroll
+  for (int a = 0; a < kFixDet; ++a) ea[a] = expo(a);
+#pragma unroll
+  for (int j = 0; j < kNBasis; ++j) eb[j] = expo(kFixDet + j);
+  eb[kNBasis] = -1;
+  if (!fits) {
+    if (threadIdx.x == 0) fix.from[blockIdx.x] = kFixNever;
+  } else {
+    // products p < 4 sqrt(2) of this tile, rounded outwards by the factor
+    {
+      uint32_t sum = 0, sq = 0;
+      float bs[kNMom];
+#pragma unroll
+      for (int j = 0; j < kNBasis; ++j) bs[j] = (float)(fabs(b[j]) * fix_pow2(-eb[j]));
+      bs[kNBasis] = 2.0f;
+#pragma unroll
+      for (int a = 0; a < kFixDet; ++a) {
+        if (a >= ev.n_det) break;
+        const float x = (float)(e[a].x * fix_pow2(-ea[a])), y = (float)(e[a].y * fix_pow2(-ea[a]));
+        const float l = sqrtf(fmaf(x, x, y * y));
+#pragma unroll
+        for (int j = 0; j < kNMom; ++j) {
+          const float p = l * bs[j];
+          const uint32_t u = __reduce_add_sync(0xffffffffu, __float2uint_ru(p * (131072.0f * (1.0f + 0x1p-20f))));
+          const uint32_t v = __reduce_add_sync(0xffffffffu, __float2uint_rd(p * p * (2097152.0f * (1.0f - 0x1p-20f))));
+          if (lane == a * kNMom + j) sum = u, sq = v;
+        }
+      }
+      if (lane < NM) sum_s[warp][lane] = sum, sq_s[warp][lane] = sq;
     }
-    for (int n = 0; n < kNMom; ++n) {
-      int be = 29 + 32;  // the basis value 1, a high limb alone
-      if (n < kNBasis) {
-        ok = ok && fit(bmax[n]);
-        be = bmax[n] > 0.0 && ok ? 60 - ilogb(bmax[n]) : 0;
+    __syncthreads();
+    if (warp == 0) {
+      // lane = moment (a, j): sum in 2^-17, squares before tile t in 2^-21
+      const int n = lane < NM ? lane : NM - 1, a = n / kNMom, j = n % kNMom;
+      uint32_t sum = 0;
+#pragma unroll
+      for (int t = 0; t < T; ++t) sum += sum_s[t][n];
+      int shift = max(0, 31 - __clz(sum | 1) - 24);  // sum < 2^(shift + 25)
+      shift = max(shift, max(__shfl_sync(0xffffffffu, shift, (lane + kNMom) % NM),
+                             __shfl_sync(0xffffffffu, shift, (lane + 2 * kNMom) % NM)));
+      int xa = 0, xb = -1;
+      uint32_t ha = 0, hb = 1;
+#pragma unroll
+      for (int i = 0; i < kFixDet; ++i)
+        if (a == i) xa = ea[i], ha = top[i];
+#pragma unroll
+      for (int i = 0; i < kNBasis; ++i)
+        if (j == i) xb = eb[i], hb = top[kFixDet + i];
+      const bool any = ha != 0 && hb != 0;  // else the products are zero, and exact
+      const int ee = ha ? 60 - xa : 0, be = hb ? 60 - xb - shift : 0;
+      const int ends = (int)((min(K - (int64_t)blockIdx.x * kFixBins, (int64_t)kFixBins) + kTileBins - 1) / kTileBins);
+      int last = 0;  // the last tile in which an end fails with nothing before the block
+      FixBlock& fc = fix.block[blockIdx.x];
+      if (lane < NM && a < ev.n_det) {
+        fc.scale[n] = fix_pow2(66 - ee - be);
+        double sq = 0.0, need = 0.0;  // in 2^(2 (xa + xb))
+#pragma unroll
+        for (int t = 0; t < T; ++t) {
+          if (any && t < ends && fix_fails(fix_pow2(shift - 54), t, sq)) {
+            need = fmax(need, fix_need(fix_pow2(shift - 54), t) - sq);
+            last = t;
+          }
+          sq += (double)sq_s[t][n] * 0x1p-21;
+        }
+        const double u = fix_pow2(2 * (xa + xb));
+        const int64_t at = (int64_t)n * gridDim.x + blockIdx.x;
+        fix.sq[at] = sq * u;
+        fix.need[at] = blockIdx.x == 0 ? 0.0 : need * u;
+        if (a == 0 && j < kNBasis) be_s[j] = be;
+        if (n == kNBasis) fc.one = 1 << (be - 32);
       }
-      for (int i = 0; i < ev.n_det; ++i)
-        if (ok && sum[i][n] > 0.0) be = min(be, 127 - ee[i] - ilogb(sum[i][n]));
-      if (n == kNBasis) {
-        ok = ok && be >= 32;
-        fc.one = ok ? 1 << (be - 32) : 0;
-      }
-      for (int i = 0; i < ev.n_det; ++i) {
-        ok = ok && abs(66 - ee[i] - be) <= 1000;
-        fc.scale[i * kNMom + n] = ldexp(1.0, ok ? 66 - ee[i] - be : 0);
-      }
-      fc.be[n] = be;
+      __syncwarp();
+      last = __reduce_max_sync(0xffffffffu, last);
+      if (lane == 0) fix.from[blockIdx.x] = blockIdx.x == 0 ? kTileBins * (last + 1) : 0;
     }
-    for (int i = 0; i < ev.n_det; ++i) fc.ee[i] = ee[i];
-    fits = ok;
-    if (!ok) atomicMax(from, kFixNever);
+    __syncthreads();
+    int4* t = fix.tile + tile * (kFixQuads * kTileBins) + lane;
+#pragma unroll
+    for (int j = 0; j < kNBasis; ++j) {
+      const Limbs l = fix_limbs_neg(__double2ll_rn(b[j] * fix_pow2(be_s[j])));
+      t[j * kTileBins] = make_int4(__double2loint(b[j]), __double2hiint(b[j]), l.h, l.l);
+    }
+#pragma unroll
+    for (int a = 0; a < kFixDet; ++a) {
+      const double u = top[a] ? fix_pow2(60 - ea[a]) : 1.0;
+      const Limbs x = fix_limbs_neg(__double2ll_rn(e[a].x * u)), y = fix_limbs_neg(__double2ll_rn(e[a].y * u));
+      t[(kNBasis + a) * kTileBins] = make_int4(x.h, x.l, y.h, y.l);
+    }
   }
+  // (the last block's reads of the others' writes go past L1)
+  __threadfence();
   __syncthreads();
-  if (!on || lane != 0) return;
-  const int n = a * kNMom + j;
-  const double unit = fc.scale[n];
-  double sq = 0.0, need = 0.0;
-  int last = 0;  // block 0: the last tile in which an end fails
-  // (products that are all zero are exact)
-#pragma unroll
-  for (int t = 0; t < T; ++t) {
-    if (s > 0.0 && fix_fails(unit, t, sq)) {
-      need = fmax(need, fix_need(unit, t) - sq);
-      last = t;
-    }
-    sq += q[t];
-  }
-  guard[blockIdx.x].sq[n] = sq;
-  guard[blockIdx.x].need[n] = blockIdx.x == 0 ? 0.0 : need;
-  if (blockIdx.x == 0) atomicMax(from, kTileBins * (last + 1));
-}
-
-// fix_from over all blocks: one CTA, a warp a moment, lanes over the blocks; an
-// exclusive prefix sum of the blocks' squares against what each needs before
-// it. *from rises past the last block that fails.
-__global__ void __launch_bounds__(kFixScaleThreads) fix_guard_kernel(int n_det, int64_t blocks, const FixGuard* guard, int* from) {
-  const int n = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (n >= n_det * kNMom) return;
-  double before = 0.0;
-  int last = -1;
-  for (int64_t g0 = 0; g0 < blocks; g0 += 32) {
-    const int64_t g = g0 + lane;
-    const double sq = g < blocks ? guard[g].sq[n] : 0.0;
-    double incl = sq;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const double x = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += x;
-    }
-    double excl = __shfl_up_sync(0xffffffffu, incl, 1);
-    excl = before + (lane ? excl : 0.0);
-    if (g < blocks && !(guard[g].need[n] <= excl)) last = (int)g;
-    before += __shfl_sync(0xffffffffu, incl, 31);
-  }
-  if (last >= 0) atomicMax(from, (last + 1) * kFixBins);
-}
-
-// One CTA per block of kStageBins bins, one thread per bin: the bin's
-// fixed-point quads (zeros past the last bin).
-__global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const FixBlock* fc, const int* from, int4* out) {
-  const int64_t K = ev.n_bins, k = (int64_t)blockIdx.x * kStageBins + threadIdx.x;
-  if (*from >= K) return;
-  const bool in = k < K;
-  const FixBlock& c = fc[k / kFixBins];
-  int4* t = out + k / kTileBins * (kFixQuads * kTileBins) + k % kTileBins;
-  for (int j = 0; j < kNBasis; ++j) {
-    const double b = in ? ev.b64[j * K + k] : 0.0;
-    const Limbs l = fix_limbs_neg((int64_t)rint(ldexp(b, c.be[j])));
-    t[j * kTileBins] = make_int4(__double2loint(b), __double2hiint(b), l.h, l.l);
-  }
-  for (int a = 0; a < kFixDet; ++a) {
-    const double2 e = in && a < ev.n_det ? ev.e64[a * K + k] : make_double2(0.0, 0.0);
-    const int s = a < ev.n_det ? c.ee[a] : 0;
-    const Limbs x = fix_limbs_neg((int64_t)rint(ldexp(e.x, s))), y = fix_limbs_neg((int64_t)rint(ldexp(e.y, s)));
-    t[(kNBasis + a) * kTileBins] = make_int4(x.h, x.l, y.h, y.l);
-  }
+  if (threadIdx.x == 0) last_s = atomicInc(fix.done, gridDim.x - 1) == gridDim.x - 1;
+  __syncthreads();
+  if (!last_s) return;
+  __threadfence();
+  fix_from_all(ev.n_det, (int)gridDim.x, fix);
 }
 
 }  // namespace sharpy
@@ -224,7 +265,7 @@ __global__ void __launch_bounds__(kStageBins) fix_tile_kernel(DevEvent ev, const
 // octant, where long double has the bits for it on every host).
 static const int4* fix_trig_host() {
   static const std::vector<int4> t = [] {
-    std::vector<int4> v(kFixTrig);
+    std::vector<int4> v(kFixTrig + 1, int4{0, 0, 0, 0});  // the count after it (FixTables::done) starts at zero
     constexpr int O = kFixTrig / 8;
     int64_t co[O + 1], si[O + 1];
     for (int i = 0; i <= O; ++i) {
@@ -244,40 +285,47 @@ static const int4* fix_trig_host() {
   return t.data();
 }
 
-// The fixed-point tables of the FP64 path, built with every data set; without
-// them (memory, too many bins, data that no scale fits) the FP64 sweep runs.
-static cudaError_t build_fixed(sharpy_ctx* c, int64_t blocks) {
+// The sweeps' tables, built with every data set (they hold E). Without the
+// fixed-point ones (memory, too many bins, data that no scale fits) the FP64
+// sweep runs.
+static cudaError_t build_tables(sharpy_ctx* c, int64_t blocks) {
   DevEvent& ev = c->ev;
   ev.tile_fix = nullptr;
   ev.fix_from = nullptr;
   ev.fix_block = nullptr;
   ev.fix_trig = nullptr;
-  if (ev.n_bins > kFixMaxBins || ev.n_det > kFixDet) return cudaSuccess;
-  const size_t tiles = (size_t)blocks * kStageBins * kFixQuads;
-  if (!c->d_fix) {
-    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig) * sizeof(int4) + (size_t)blocks * (sizeof(FixBlock) + sizeof(FixGuard)) +
-                                  sizeof(int)) != cudaSuccess) {
+  float4* split = c->d_tile + blocks * (stage_bytes(false) / 16);
+  const size_t tiles = (size_t)blocks * kStageBins * kFixQuads, rule = (size_t)blocks * kFixDet * kNMom;
+  if (!c->d_fix && ev.n_bins <= kFixMaxBins && ev.n_det <= kFixDet) {
+    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig + 1) * sizeof(int4) + (size_t)blocks * (sizeof(FixBlock) + sizeof(int)) +
+                                  2 * rule * sizeof(double) + sizeof(int)) != cudaSuccess) {
       c->d_fix = nullptr;
       (void)cudaGetLastError();
-      return cudaSuccess;
+    } else {
+      const cudaError_t e = cudaMemcpy(c->d_fix + tiles, fix_trig_host(), (kFixTrig + 1) * sizeof(int4), cudaMemcpyHostToDevice);
+      if (e != cudaSuccess) return e;
     }
-    const cudaError_t e = cudaMemcpy(c->d_fix + tiles, fix_trig_host(), kFixTrig * sizeof(int4), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return e;
   }
-  FixBlock* fc = reinterpret_cast<FixBlock*>(c->d_fix + tiles + kFixTrig);
-  FixGuard* guard = reinterpret_cast<FixGuard*>(fc + blocks);
-  int* from = reinterpret_cast<int*>(guard + blocks);
-  cudaError_t e = cudaMemset(from, 0, sizeof(int));
+  FixTables fix{};
+  if (c->d_fix) {
+    fix.tile = c->d_fix;
+    fix.done = reinterpret_cast<unsigned int*>(c->d_fix + tiles + kFixTrig);
+    fix.block = reinterpret_cast<FixBlock*>(c->d_fix + tiles + kFixTrig + 1);
+    fix.sq = reinterpret_cast<double*>(fix.block + blocks);
+    fix.need = fix.sq + rule;
+    fix.from = reinterpret_cast<int*>(fix.need + rule);
+  }
+  event_tables_kernel<<<(unsigned)blocks, kStageBins>>>(ev, c->d_tile, split, fix);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  fix_scale_kernel<<<(unsigned)blocks, kFixScaleThreads>>>(ev, fc, guard, from);
-  fix_guard_kernel<<<1, kFixScaleThreads>>>(ev.n_det, blocks, guard, from);
-  fix_tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, fc, from, c->d_fix);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  ev.tile_fix = c->d_fix;
-  ev.fix_from = from;
-  ev.fix_block = fc;
-  ev.fix_trig = c->d_fix + tiles;
+  ev.tile_mixed = c->d_tile;
+  ev.tile_split = split;
+  if (c->d_fix) {
+    ev.tile_fix = fix.tile;
+    ev.fix_from = fix.from + blocks;
+    ev.fix_block = fix.block;
+    ev.fix_trig = c->d_fix + tiles;
+  }
   return cudaSuccess;
 }
 
@@ -457,17 +505,39 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   }
   const std::vector<double>& amp = c->h_amp;
   std::vector<double> e64(2 * n_det * K), pref(n_det * K), wamp2(n_det * K);
+  // E = w conj(d) f^-7/6, from which the device makes the sweeps' tables while
+  // the host goes on
+  for (int a = 0; a < n_det; ++a)
+    for (int64_t k = 0; k < K; ++k) {
+      const int64_t i = a * K + k;
+      const double w = 4.0 * df / psd[i];
+      wamp2[i] = w;
+      e64[2 * i] = w * d[2 * i] * amp[k];
+      e64[2 * i + 1] = -w * d[2 * i + 1] * amp[k];
+    }
+  DevEvent& ev = c->ev;
+  ev.n_det = n_det;
+  ev.n_bins = K;
+  ev.f_min = f_min;
+  ev.df = df;
+  ev.inv_df = 1.0 / df;
+  ev.f = c->d_f;
+  ev.b64 = c->d_b64;
+  ev.e64 = c->d_e64;
+  ev.pref = c->d_pref;
+  if (cudaMemcpy(c->d_e64, e64.data(), e64.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+      build_tables(c, blocks) != cudaSuccess) {
+    free_event(c);
+    return SHARPY_ECUDA;
+  }
   // <d|d> with a compensated sum; P_a prefix sums of w f^-7/3 (compensated).
   double dd = 0.0, ddc = 0.0;
   for (int a = 0; a < n_det; ++a) {
     double s = 0.0, cmp = 0.0;
     for (int64_t k = 0; k < K; ++k) {
       int64_t i = a * K + k;
-      double w = 4.0 * df / psd[i];
+      double w = wamp2[i];
       double dr = d[2 * i], di = d[2 * i + 1];
-      // E = w conj(d) f^-7/6
-      e64[2 * i] = w * dr * amp[k];
-      e64[2 * i + 1] = -w * di * amp[k];
       double term = w * amp[k] * amp[k];
       wamp2[i] = term;
       double t = s + term;
@@ -480,12 +550,6 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
       dd = u;
     }
   }
-  const bool ok = cudaMemcpy(c->d_e64, e64.data(), e64.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess &&
-                  cudaMemcpy(c->d_pref, pref.data(), pref.size() * sizeof(double), cudaMemcpyHostToDevice) == cudaSuccess;
-  if (!ok) {
-    free_event(c);
-    return SHARPY_ECUDA;
-  }
   // the Fisher prefix tables depend on w f^-7/3 only: kept while it is unchanged
   if (wamp2 != c->h_wamp2) {
     cudaFree(c->d_p1);
@@ -493,34 +557,20 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
     c->d_p1 = c->d_p2 = nullptr;
     c->h_wamp2.swap(wamp2);
   }
-  DevEvent& ev = c->ev;
-  ev.n_det = n_det;
-  ev.n_bins = K;
-  ev.f_min = f_min;
-  ev.df = df;
-  ev.inv_df = 1.0 / df;
   ev.dd = dd + ddc;
   {
     const double h = -0.5 * ev.dd;  // the epilogue's starting sum, as a double-float
     ev.ddh_hi = (float)h;
     ev.ddh_lo = (float)(h - (double)ev.ddh_hi);
   }
-  ev.f = c->d_f;
-  ev.b64 = c->d_b64;
-  ev.e64 = c->d_e64;
-  ev.pref = c->d_pref;
   ev.p1 = c->d_p1;
   ev.p2 = c->d_p2;
   for (int a = 0; a < n_det; ++a) detector_geometry(det[a], ev.det[a]);
-  // the sweeps' tiles (rebuilt with every data set: they hold E)
-  float4* split = c->d_tile + blocks * (stage_bytes(false) / 16);
-  tile_kernel<<<(unsigned)blocks, kStageBins>>>(ev, c->d_tile, split);
-  if (cudaGetLastError() != cudaSuccess || build_fixed(c, blocks) != cudaSuccess || cudaDeviceSynchronize() != cudaSuccess) {
+  if (cudaMemcpy(c->d_pref, pref.data(), pref.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaDeviceSynchronize() != cudaSuccess) {
     free_event(c);
     return SHARPY_ECUDA;
   }
-  ev.tile_mixed = c->d_tile;
-  ev.tile_split = split;
   c->has_data = true;
   return SHARPY_OK;
 }

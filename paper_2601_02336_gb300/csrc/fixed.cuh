@@ -19,7 +19,7 @@
 //   data    E scaled to 2^61 by the block's largest;
 //   moments sums of the products' high words: exact, in any order, up to the
 //           block's final rounding to FP64 (FP64 sweep: one rounding per bin).
-// Scales are powers of two per block of 256 bins (fix_scale_kernel): over so
+// Scales are powers of two per block of 256 bins (event_tables_kernel): over so
 // few bins E and the basis change little, and their sums need few bits of
 // headroom (with blocks of 2048 a sweep that ends early had up to 30 times the
 // FP64 sweep's error).
@@ -56,19 +56,12 @@ constexpr int kFixTrig = 1024;            // points of the carrier table, {cos h
 // A block's scales: moment (a, j) = scale[a * kNMom + j] x integer sum.
 struct FixBlock {
   double scale[kFixDet * kNMom];
-  int one;             // high limb of the basis value 1
-  int ee[kFixDet];     // E_a's limbs: 2^ee E_a
-  int be[kNMom];       // B_j's: 2^be B_j
+  int one;  // high limb of the basis value 1
 };
 
-// What a block's moment (a, j) brings to the rule above: the sum of squares of
-// its products, and what those of all earlier blocks must reach at least so that
-// no end in the block fails.
-struct FixGuard {
-  double sq[kFixDet * kNMom], need[kFixDet * kNMom];
-};
 // Whether a sweep that ends in tile t of a block fails: `unit` of the block's
-// moment, `sq` of the products of all bins before the tile.
+// moment, `sq` the sum of squares of its products in all bins before the tile,
+// which must reach fix_need.
 __host__ __device__ __forceinline__ double fix_need(double unit, int t) {
   const double u = unit * 0x1p49;  // a unit in 16 roundings of FP64 to 1
   return u * u * (double)(kTileBins * (t + 1));

@@ -446,3 +446,22 @@ def test_loglike_fp64_data_without_a_scale():
     assert torch.allclose(big * 2.0 ** -300, l, rtol=1e-12, atol=0.0)
     assert torch.allclose(gbig * 2.0 ** -300, g, rtol=1e-9, atol=1e-9 * float(g.abs().max()))
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("block", [1, 31, 32, 700, 1013])
+def test_fixed_point_rule_over_many_blocks(block):
+    """The rule on the sweeps' ends is formed over all blocks of a segment (1014 here) by the CTA that comes last: a
+    bin 2^20 times too large sends the sweeps that end before the end of its block to FP64; the same grid with
+    ordinary data again from the first tile on."""
+    G.require_gpu()
+    w = inputs.bns()
+    ctx = api.Context.from_workload(w)
+    psd, dets = inputs.psd_array(w), inputs.detectors(w)
+    d0 = inputs.noise(w, 3)
+    for a in range(w.n_det):
+        d = d0.copy()
+        ctx.set_data(d, psd, w.f_min, w.df, dets)
+        assert ctx.fixed_point_from() == 32
+        d[a, block * 256 + 17 * a] *= 2.0 ** 20
+        ctx.set_data(d, psd, w.f_min, w.df, dets)
+        assert ctx.fixed_point_from() == min((block + 1) * 256, w.n_bins)
