@@ -18,6 +18,7 @@
 
 #include "context.cuh"
 #include "physics.cuh"
+#include "quotient.cuh"
 
 using namespace sharpy;
 
@@ -66,23 +67,6 @@ struct MetricShared {
   double piv[kMetPad], rpiv[kMetPad];
   unsigned ok[2];                      // per particle: the factorisation of M, of M^-1 went through
 };
-
-// t / c from c's correctly rounded reciprocal r (Markstein, IBM J. Res. Dev.
-// 34, 1990): with q within an ulp of t / c, q + (t - q c) r in fused operations
-// is the correctly rounded quotient, the bits of t / c. The first step brings
-// q = t r there, the second rounds: 5 operations that share one reciprocal
-// over a column. Outside the exponent range where that holds it divides.
-__device__ __forceinline__ double quotient(double t, double c, double r) {
-  const int ht = __double2hiint(t) & 0x7fffffff, hr = __double2hiint(r) & 0x7fffffff;
-  const double q = t * r;
-  const int hq = __double2hiint(q) & 0x7fffffff;
-  constexpr int lo = 200 << 20, hi = 1846 << 20;
-  if ((ht > lo && ht < hi && hr > lo && hr < hi && hq > lo && hq < hi) || (ht | __double2loint(t)) == 0) {
-    const double q1 = __fma_rn(__fma_rn(-q, c, t), r, q);
-    return __fma_rn(__fma_rn(-q1, c, t), r, q1);
-  }
-  return t / c;
-}
 
 // The phase derivative's basis coefficients D_j: parameters 0..3 (masses and
 // spins) have the eight post-Newtonian terms and the constant, phi_c the

@@ -72,3 +72,22 @@ def test_local_metric_block_edges(name, n):
     guard = torch.full((n + 1, w.n_dim, w.n_dim), -7.0, dtype=torch.float64, device="cuda")
     rc = api.lib().sharpy_local_metric(ctx._h, n, api._ptr(th), 0.6, None, api._ptr(guard), None, api._stream())
     assert rc == 0 and torch.equal(guard[:n], full["inv_mass"][:n]) and bool((guard[n] == -7.0).all())
+
+
+@pytest.mark.parametrize("dim", [0, 1, 2])
+def test_local_metric_infinite_precision(dim):
+    """A component so narrow that its precision overflows: the factorisation fails, the diagonal stays, and that
+    dimension's inverse mass is 0 without touching the others."""
+    G.require_gpu()
+    sig = [0.1, 0.2, 0.3]
+    lo, hi, mu = [-1.0] * 3, [1.0] * 3, [[0.0] * 3]
+    at = G.to_dev(np.zeros((33, 3)))
+    want = api.Context(api.gaussmix_config(lo, hi, [0.0], mu, [sig])).local_metric(at, 1.0)
+    sig[dim] = 1e-160
+    got = api.Context(api.gaussmix_config(lo, hi, [0.0], mu, [sig])).local_metric(at, 1.0)
+    for k in ("inv_mass", "chol"):
+        ref = want[k].clone()
+        ref[:, dim, :] = 0.0
+        ref[:, :, dim] = 0.0
+        assert torch.allclose(got[k], ref, rtol=1e-14, atol=0.0), k
+    assert torch.isinf(got["mass"][:, dim, dim]).all()
