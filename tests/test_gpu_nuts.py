@@ -386,3 +386,42 @@ def test_nuts_geometry_invariant(n):
             ref = ref or got
             assert all(torch.equal(a, b) for a, b in zip(got, ref)), (prec, slots)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("metric", ["identity", "local"])
+@pytest.mark.parametrize("name,n_det,n", [("tiny", 1, 1), ("tiny", 1, 9), ("tiny", 1, 33), ("bbh11", 1, 35),
+                                          ("bbh11", 2, 33), ("bbh11", 3, 9), ("bbh11", 3, 131),
+                                          ("tiny", 1, 4 * 2 * 152), ("tiny", 1, 4 * 2 * 152 + 1)])
+def test_nuts_fp64_slot_count_invariant(name, n_det, n, metric):
+    """On the FP64 path a slot's prologue runs on four lanes in tasks of eight slots and its epilogue on a group of 16,
+    8 or 4 lanes, as the slots per CTA (4, 8, 16, 32, or the call's own choice) give. Particles and statistics are the
+    same bit for bit, with ragged last CTAs, one to three detectors, sweeps that end before the fixed-point bins begin
+    or have no bins at all, and both kinds of metric; the ln L and gradient that come back are the likelihood call's at
+    the returned positions."""
+    G.require_gpu()
+    w = inputs.WORKLOADS[name]()
+    if name == "bbh11":
+        w.n_det, w.f_min, w.n_bins = n_det, 40.0, 700
+    ctx, th_inj, _ = api.make_event(w, seed=0)
+    th = inputs.prior_draws(w, n, 61)
+    th[n // 2:] = inputs.ball(w, th_inj, n - n // 2, 62)
+    t0 = G.to_dev(th)
+    l0, g0 = ctx.loglike_grad(t0, "fp64")
+    m = ctx.local_metric(t0, 0.3)
+    ref = None
+    for slots in (0, 4, 8, 16, 32):
+        ctx.set_nuts_slots(slots)
+        t, l, g = t0.clone(), l0.clone(), g0.clone()
+        if metric == "identity":
+            st = ctx.nuts_mutate(0.3, t, l, g, None, 1e-3, 4, 2, key=5, ctr=9, precision="fp64")
+        else:
+            st = ctx.nuts_mutate_local(0.3, t, l, g, m["inv_mass"], m["chol"], 0.2, 4, 2, key=5, ctr=9,
+                                       precision="fp64")
+        got = (t, l, g, st)
+        ref = ref or got
+        assert all(torch.equal(a, b) for a, b in zip(got, ref)), slots
+    assert n == 1 or not torch.equal(ref[0], t0)  # one particle may reject both transitions
+    lc, gc = ctx.loglike_grad(ref[0], "fp64")
+    live = torch.isfinite(lc)
+    assert torch.equal(lc[live], ref[1][live]) and torch.equal(gc[live], ref[2][live])
+    ctx.clear_status()
