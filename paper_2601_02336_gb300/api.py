@@ -136,7 +136,7 @@ class Context:
 
     def set_loglike_split(self, split):
         """Force 1, 2, 4 or 8 warps per vector, or 16 (the staged kernel of long segments, mixed and split
-        paths; 8 where it does not apply), in later likelihood calls (0: tune)."""
+        paths; 8 where it does not apply), in later likelihood calls (0: tune). FP64: 8 and 16 are 4."""
         check(lib().sharpy_set_loglike_split(self._h, int(split)), "sharpy_set_loglike_split")
 
     def set_nuts_slots(self, slots):

@@ -107,10 +107,11 @@ static int launch_ll(sharpy_ctx* c, int64_t n, const double* th, double* lnl, do
   for (const auto& e : c->ll_tuned)
     if (e.key == key) return launch_ll_prec<PREC, GRAD>(c, e.split, n, th, lnl, grad, s) == cudaSuccess
                                  ? SHARPY_OK : SHARPY_ECUDA;
-  // 1, 2, 4, 8 warps per vector, and the staged kernel where it applies
+  // 1, 2, 4, 8 warps per vector (as many as a CTA has), and the staged kernel where it applies
   TuneCandidate cands[kNumSplitChoices + 1];
   int nc = 0;
-  for (int i = 0; i < kNumSplitChoices; ++i) cands[nc++].slots = kSplitChoices[i];
+  for (int i = 0; i < kNumSplitChoices; ++i)
+    if (kSplitChoices[i] <= ll_warps(PREC)) cands[nc++].slots = kSplitChoices[i];
   if (PREC != SHARPY_FP64 && c->ev.n_bins >= kStageMinBins) cands[nc++].slots = kSplitStaged;
   auto trial = [&](int split, cudaStream_t ts) -> int {
     return launch_ll_prec<PREC, GRAD>(c, split, n, th, lnl, grad, ts) == cudaSuccess ? SHARPY_OK : SHARPY_ECUDA;

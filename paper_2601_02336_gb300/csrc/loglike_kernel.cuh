@@ -338,12 +338,14 @@ inline cudaError_t launch_ll_split(sharpy_ctx* c, int split, int64_t n, const do
     if constexpr (PREC == SHARPY_MIXED_SPLIT) {
       if (c->ev.n_bins >= kStageMinBins) return launch_ll_staged_split_unit(c, GRAD, NDET, n, th, lnl, grad, s);
     }
-    split = 8;  // no staged tables, or the FP64 path: all warps of a CTA
+    split = 8;  // a short segment, or the FP64 path: all warps of a CTA
   }
   switch (split) {
     case 2: launch_ll_one<PREC, GRAD, NDET, 2>(c, n, th, lnl, grad, s); break;
     case 4: launch_ll_one<PREC, GRAD, NDET, 4>(c, n, th, lnl, grad, s); break;
-    case 8: launch_ll_one<PREC, GRAD, NDET, ll_warps(PREC)>(c, n, th, lnl, grad, s); break;
+    case 8:  // all warps of a CTA: eight, four on the FP64 path (the kernel of choice 4)
+      launch_ll_one<PREC, GRAD, NDET, ll_warps(PREC)>(c, n, th, lnl, grad, s);
+      break;
     default: launch_ll_one<PREC, GRAD, NDET, 1>(c, n, th, lnl, grad, s); break;
   }
   return cudaGetLastError();

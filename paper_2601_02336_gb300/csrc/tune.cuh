@@ -19,8 +19,9 @@ namespace sharpy {
 
 constexpr int kSlotChoices[] = {4, 8, 16, 32};
 constexpr int kNumSlotChoices = 4;
-// Warps that share one particle's sweep in the standalone likelihood kernel
-// (plus the staged kernel, choice 16, on long segments of the mixed path).
+// Warps that share one particle's sweep in the standalone likelihood kernel (at
+// most those of a CTA, four on the FP64 path), plus the staged kernel, choice 16,
+// on long segments of the mixed and split paths.
 constexpr int kSplitChoices[] = {1, 2, 4, 8};
 constexpr int kNumSplitChoices = 4;
 

@@ -465,3 +465,20 @@ def test_fixed_point_rule_over_many_blocks(block):
         d[a, block * 256 + 17 * a] *= 2.0 ** 20
         ctx.set_data(d, psd, w.f_min, w.df, dets)
         assert ctx.fixed_point_from() == min((block + 1) * 256, w.n_bins)
+
+
+def test_loglike_fp64_tuner_choices():
+    """The FP64 path's CTAs have four warps: its tuner times 1, 2 and 4 warps per vector and reports one of them; the
+    forced choices 8 and 16 stay accepted and give the same results."""
+    G.require_gpu()
+    w = inputs.bbh11()
+    ctx, th_inj, _ = api.make_event(w, seed=0)
+    for n in (1, 7, 64, 300, 1000):
+        th = G.to_dev(inputs.ball(w, th_inj, n, 70 + n))
+        l, g = ctx.loglike_grad(th, "fp64")
+        assert ctx.loglike_split(n, "fp64") in (1, 2, 4)
+        for split in (4, 8, 16):
+            ctx.set_loglike_split(split)
+            lf, gf = ctx.loglike_grad(th, "fp64")
+            assert torch.equal(lf, l) and torch.equal(gf, g), (n, split)
+        ctx.set_loglike_split(0)
