@@ -14,8 +14,10 @@
 // word of a product is ah bh + (ah bl + al bh) / 2^32, rounded: 3 multiply-adds,
 // error under one unit. Errors against the FP64 sweep's, per bin:
 //   phase   the same FP64 sum, then its fraction of a turn exact to 2^-64;
-//   carrier within 2^-58 (a table of 1024 points to 2^-62, sine and cosine of
-//           the rest, |d| <= pi / 1024, by their Taylor series); FP64: 2^-53;
+//   carrier E times it within 2^-56.5 of the block's largest |E| (2^-59.5 rms a
+//           part; a table of 1024 points to 2^-62, sine and cosine of the rest,
+//           |d| <= pi / 1024, by their Taylor series: 2^-57.3 and 2^-59.5 at
+//           its ends); FP64: 2^-53 of |E|;
 //   data    E scaled to 2^61 by the block's largest;
 //   moments sums of the products' high words: exact, in any order, up to the
 //           block's final rounding to FP64 (FP64 sweep: one rounding per bin).
@@ -157,7 +159,7 @@ constexpr uint32_t kFixB1 = (uint32_t)(147573952589676412928.0 * kFixKappa * kFi
 
 // sin d and cos d - 1 in units of 2^-64:
 //   sin d     = (pi / 1024) y (1 - kappa y^2 / 6 + kappa^2 y^4 / 120)   (next term 2^-70)
-//   cos d - 1 = -(kappa y^2 / 2) (1 - kappa y^2 / 12)                   (next term 2^-59.3)
+//   cos d - 1 = -(kappa y^2 / 2) (1 - kappa y^2 / 12)                   (next term 2^-59.6)
 // The brackets' corrections, 2^-19 and below, need y^2 to 31 bits only.
 __host__ __device__ __forceinline__ void fix_small(int64_t rest, int64_t* s, int64_t* c1) {
   const Limbs v = fix_limbs(rest);

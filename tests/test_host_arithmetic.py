@@ -1,6 +1,7 @@
 """Device arithmetic that is plain C++ (host and device functions of the csrc headers), compiled for the host and
 compared with wider or plainer arithmetic. No GPU."""
 import os
+import platform
 import shutil
 import subprocess
 
@@ -29,3 +30,15 @@ def test_quotient_has_the_bits_of_the_division(tmp_path, seed):
     takes the fused steps, zeros of both signs, subnormals, infinities and NaN as numerator and divisor."""
     (n, bad), err = _run(tmp_path, "quotient_check.cpp", seed)
     assert int(n) > 4_000_000 and int(bad) == 0, err
+
+
+@pytest.mark.parametrize("seed", [1, 2])
+def test_fixed_point_functions(tmp_path, seed):
+    """fixed.cuh's fraction of a turn, sine and cosine of the rest, carrier and moment sums against 113-bit arithmetic,
+    each within the bound that the check derives, index wraps, the rest's ends and limb boundaries included."""
+    out, _ = _run(tmp_path, "fixed_point_check.cpp", seed, libs=["-lquadmath"] if platform.machine() == "x86_64" else [])
+    rows = {out[i]: (float(out[i + 1]), float(out[i + 2])) for i in range(0, len(out), 3)}
+    assert set(rows) == {"limbs", "frac", "index_and_rest", "sine", "cosine", "carrier", "carrier_rms_per_part",
+                         "moment_per_product", "moment_of_one_per_product"}
+    for name, (worst, bound) in rows.items():
+        assert worst <= bound, name
