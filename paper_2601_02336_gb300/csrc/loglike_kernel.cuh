@@ -106,24 +106,24 @@ loglike_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restrict__ th
       fin = fin && isfinite(g);
     }
     if (!fin) set_status(status, SHARPY_ENONFINITE);
-    return;
-  }
-  __syncthreads();
-  if (warp == 0 && lane < PPC) {
-    int64_t q = base + lane;
-    if (q < n) {
-      double l = NAN, gph[SHARPY_NPHYS];
-      if (sc[lane].ok) epilogue<DT, GRAD>(ev, sc[lane], ec[lane], mom[lane], &l, gph);
-      lnl[q] = l;
-      bool fin = isfinite(l);
-      if (GRAD) {
-        for (int i = 0; i < D; ++i) {
-          double g = sc[lane].ok ? gph[m.phys[i]] : NAN;
-          grad[q * D + i] = g;
-          fin = fin && isfinite(g);
+  } else {
+    __syncthreads();
+    if (warp == 0 && lane < PPC) {
+      int64_t q = base + lane;
+      if (q < n) {
+        double l = NAN, gph[SHARPY_NPHYS];
+        if (sc[lane].ok) epilogue<GRAD>(ev, sc[lane], ec[lane], mom[lane], &l, gph);
+        lnl[q] = l;
+        bool fin = isfinite(l);
+        if (GRAD) {
+          for (int i = 0; i < D; ++i) {
+            double g = sc[lane].ok ? gph[m.phys[i]] : NAN;
+            grad[q * D + i] = g;
+            fin = fin && isfinite(g);
+          }
         }
+        if (!fin) set_status(status, SHARPY_ENONFINITE);
       }
-      if (!fin) set_status(status, SHARPY_ENONFINITE);
     }
   }
 }
@@ -287,7 +287,7 @@ loglike_staged_kernel(DevModel m, DevEvent ev, int64_t n, const double* __restri
     const int64_t q = base + lane;
     if (q < n) {
       double l = NAN, gph[SHARPY_NPHYS];
-      if (sc[lane].ok) epilogue<float, GRAD>(ev, sc[lane], ec[lane], mom[lane], &l, gph);
+      if (sc[lane].ok) epilogue<GRAD>(ev, sc[lane], ec[lane], mom[lane], &l, gph);
       lnl[q] = l;
       bool fin = isfinite(l);
       if (GRAD) {

@@ -1019,7 +1019,7 @@ __global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
             gph = SM.gph[cs];
             __syncwarp(gmask);
           } else {
-            epilogue<DT, true>(A.ev, sc[cs], ec[cs], mom[cs], &sl.lnl_new, gown);
+            epilogue<true>(A.ev, sc[cs], ec[cs], mom[cs], &sl.lnl_new, gown);
           }
           sl.st_bins += (long long)(sc[cs].kisco + 1) * A.ev.n_det;
         }

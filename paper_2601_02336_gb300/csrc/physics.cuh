@@ -599,39 +599,33 @@ __device__ __forceinline__ void prologue_cta(int warp, int lane, int n, const De
 
 // Moments layout: mom[a][j][re/im], j = 0..8 basis (8 = f), j = 9 plain sum Z.
 
-// ln L (FP64 total) and d lnL / d(physical parameters) from the moments.
-// The gradient is contracted on the amplitude-scaled moments A0 Z, A0 Y_j and
-// the scaled prefix sum A0^2 P, which are O(SNR^2) and fit FP32 (the raw moments
-// and prefix sums span ~1e-22..1e43). FP64 path: ln L assembled in FP64 from
-// the raw moments. Mixed paths: from the same scaled FP32 quantities with exact
-// products and double-float sums (the moments are FP32 anyway), so only the
-// scaling A0^2 P and the conversions remain FP64.
-template <class DT, bool GRAD, class MT, class GT>
-__device__ void epilogue(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<DT>& ec, const MT* mom, double* lnl,
-                         GT* gph) {
-  constexpr bool kDF = std::is_same<DT, float>::value;
-  double acc = -0.5 * ev.dd;
-  DF accf = kDF ? DF{ev.ddh_hi, ev.ddh_lo} : DF{0.0f, 0.0f};  // = df_from(acc), formed when the data were set
+// ln L (FP64 total) and d lnL / d(physical parameters) from the moments, mixed
+// paths (the FP64 path's is epilogue_lanes below). The gradient is contracted
+// on the amplitude-scaled moments A0 Z, A0 Y_j and the scaled prefix sum A0^2 P,
+// which are O(SNR^2) and fit FP32 (the raw moments and prefix sums span
+// ~1e-22..1e43), ln L is assembled from them with exact products and
+// double-float sums (the moments are FP32 anyway), so only the scaling A0^2 P
+// and the conversions remain FP64.
+template <bool GRAD, class GT>
+__device__ void epilogue(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<float>& ec, const float* mom,
+                         double* lnl, GT* gph) {
+  using DT = float;
+  DF accf = {ev.ddh_hi, ev.ddh_lo};  // -<d|d> / 2, formed when the data were set
   DT g[SHARPY_NPHYS];
 #pragma unroll
   for (int i = 0; i < SHARPY_NPHYS; ++i) g[i] = DT(0);
   const DT a0 = ec.a0;
   for (int a = 0; a < ev.n_det; ++a) {
-    const MT* M = mom + a * kNMom * 2;
+    const float* M = mom + a * kNMom * 2;
     const double P = sc.kisco >= 0 ? ev.pref[(int64_t)a * ev.n_bins + sc.kisco] : 0.0;
     const DT cr = ec.cre[a], ci = ec.cim[a];
     const DT ps = (DT)(ec.A0sq * P);                   // A0^2 P
-    const DT zr = a0 * (DT)M[18], zi = a0 * (DT)M[19];  // A0 Z
-    if constexpr (kDF) {
-      // Re(C A0 Z) - |C|^2 A0^2 P / 2
-      const DF re = df_two_prod(cr, zr) - df_two_prod(ci, zi);
-      const DF c2 = df_two_prod(cr, cr) + df_two_prod(ci, ci);
-      const DF c2p = df_two_prod(c2.hi, 0.5f * ps) + DF{__fmul_rn(c2.lo, 0.5f * ps), 0.0f};
-      accf = accf + (re - c2p);
-    } else {
-      const double Gr = ec.A0 * (double)ec.cre[a], Gi = ec.A0 * (double)ec.cim[a];
-      acc += (Gr * (double)M[18] - Gi * (double)M[19]) - 0.5 * (Gr * Gr + Gi * Gi) * P;
-    }
+    const DT zr = a0 * M[18], zi = a0 * M[19];  // A0 Z
+    // Re(C A0 Z) - |C|^2 A0^2 P / 2
+    const DF re = df_two_prod(cr, zr) - df_two_prod(ci, zi);
+    const DF c2 = df_two_prod(cr, cr) + df_two_prod(ci, ci);
+    const DF c2p = df_two_prod(c2.hi, 0.5f * ps) + DF{__fmul_rn(c2.lo, 0.5f * ps), 0.0f};
+    accf = accf + (re - c2p);
     if (!GRAD) continue;
     const DT tp = DT(kTwoPi);
     // Im(C X) for a scaled phase-derivative moment X
@@ -641,8 +635,8 @@ __device__ void epilogue(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<
     DT yr[kNPn], yi[kNPn];
 #pragma unroll
     for (int j = 0; j < kNPn; ++j) {
-      yr[j] = a0 * (DT)M[2 * j];
-      yi[j] = a0 * (DT)M[2 * j + 1];
+      yr[j] = a0 * M[2 * j];
+      yi[j] = a0 * M[2 * j + 1];
     }
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
@@ -659,13 +653,13 @@ __device__ void epilogue(const DevEvent& ev, const SweepCoef& sc, const EpiCoef<
     g[SHARPY_DL] += ec.rel_dl * amp;
     g[SHARPY_COSI] += resp(ec.dcre[a][0], ec.dcim[a][0]);
     g[SHARPY_PSI] += resp(ec.dcre[a][1], ec.dcim[a][1]);
-    const DT yfr = a0 * (DT)M[16], yfi = a0 * (DT)M[17];
+    const DT yfr = a0 * M[16], yfi = a0 * M[17];
     g[SHARPY_RA] += resp(ec.dcre[a][2], ec.dcim[a][2]) + tp * imcx(ec.dtau[a][0] * yfr, ec.dtau[a][0] * yfi);
     g[SHARPY_SINDEC] += resp(ec.dcre[a][3], ec.dcim[a][3]) + tp * imcx(ec.dtau[a][1] * yfr, ec.dtau[a][1] * yfi);
     g[SHARPY_TC] += tp * imcx(yfr, yfi);
     g[SHARPY_PHIC] += -imcx(zr, zi);
   }
-  *lnl = kDF ? df_to_double(accf) : acc;
+  *lnl = df_to_double(accf);
   if (GRAD)
 #pragma unroll
     for (int i = 0; i < SHARPY_NPHYS; ++i) gph[i] = (GT)g[i];
