@@ -6,9 +6,10 @@
 // are reused); a bin and detector of the FP64 sweep takes about 50 of the former
 // (a third in sincospi, two fifths in the moments), or 4 of them and about 170
 // integer instructions as below. 1000 vectors near the injection (8033 bins,
-// ~320 active), with the gradient: 166 to 70 us; a NUTS mutation of 1001
-// particles 22.0 to 11.6 ms; ln L and gradient as far from a 64-bit evaluation as
-// before (4.8e-13: the phase's rounding).
+// ~320 active), with the gradient: 166 to 70 us by this alone, a NUTS mutation
+// of 1001 particles 22.0 to 11.6 ms (173 to 53 us and 21.3 to 9.1 ms with the
+// prologue and epilogue on lanes, in another event); ln L and gradient as far
+// from a 64-bit evaluation as before (1e-13 to 8e-13: the phase's rounding).
 //
 // Numbers are 64-bit integers v = h 2^32 + l with both limbs signed; the high
 // word of a product is ah bh + (ah bl + al bh) / 2^32, rounded: 3 multiply-adds,

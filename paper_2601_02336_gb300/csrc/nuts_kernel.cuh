@@ -932,7 +932,7 @@ __global__ void __launch_bounds__(W * 32, nuts_ctas<PREC, SLOTS, W>())
     }
     if (warp == cw) {
       // this tick's state machines, one per warp before a second one on any
-      // warp: pending slot of rank i goes to group (i mod 4) SPW + i / 4
+      // warp: pending slot of rank i goes to group (i mod W) SPW + i / W
       const bool pd = lane < SLOTS && S.pending[lane];
       const unsigned pm = __ballot_sync(0xffffffffu, pd);
       if (lane < SLOTS) S.cslot[lane] = -1;

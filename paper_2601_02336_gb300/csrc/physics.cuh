@@ -558,9 +558,9 @@ __device__ __forceinline__ void prologue_cta(int warp, int lane, int n, const De
                                              Pos&& pos, SweepCoef* sc, EpiCoef<DT>* ec) {
   double th[kMaxDim];
   if constexpr (std::is_same<DT, double>::value) {
-    // FP64, at most 8 particles, three warps: an instruction takes 60 cycles
-    // however many lanes are on (the phase still takes 25 thousand), so the lanes of a particle share the phase's directions and
-    // the detectors
+    // FP64, at most 4 particles, three warps: an instruction takes 60 cycles
+    // however many lanes are on (the phase still takes 25 thousand), so the
+    // lanes of a particle share the phase's directions and the detectors
     const int p = lane >> 2, i = lane & 3;
     if (warp > 2 || p >= n || (warp == 1 && i > 0) || (warp == 2 && i >= ev.n_det)) return;
     const bool on = pos(p, th);

@@ -1,15 +1,15 @@
 // The per-bin sweep: one warp accumulates the moments of one particle.
 //
-// Lane l visits bins k = l, l+32, ... <= k_ISCO (the mixed paths read tiles of
-// 32 bins, common.cuh; the FP64 path SoA tables).
+// Lane l visits bins k = l, l+32, ... <= k_ISCO, in tiles of 32 bins (common.cuh,
+// fixed.cuh; the FP64 sweep reads SoA tables).
 // Per bin the phase polynomial sum_j alpha_j B_j(f_k) + c0 is shared by all
 // detectors; per detector it adds f_k tau_a, reduces mod 1 turn, forms the
 // carrier e^{-i Psi}, multiplies the pre-whitened data E_ak and accumulates
 // Z_a (and, for the gradient, Y_aj = sum z B_j).
 //
 //   SHARPY_FP64  : the phase in FP64; carrier, data product and moments in
-//                  64-bit fixed point (fixed.cuh: errors below FP64's), or, for
-//                  data and ends that it does not fit, FP64 throughout (reduction
+//                  64-bit fixed point, or, for the data and ends where that
+//                  would lose bits (fixed.cuh), FP64 throughout (reduction
 //                  Psi - rint(Psi); sincospi).
 //   SHARPY_MIXED_SPLIT : as SHARPY_MIXED, but the phase polynomial is built
 //                  from hi/lo FP32 splits of alpha_j, tau_a and B_j(f_k):

@@ -3,9 +3,9 @@
 // caller's own call; its results do not depend on the split either.
 //
 // Autotuner for the persistent NUTS launch: the slot count (particles per
-// CTA, i.e. the CTA's tile of particles) trades the FP64 cost of the per-
-// particle phases, which warp 0 runs with one lane per slot, against the
-// number of CTAs that fill the SMs. Which one wins depends on N, the segment
+// CTA, i.e. the CTA's tile of particles) trades the cost of the per-particle
+// phases, which the slots of a CTA share by lanes, against the number of CTAs
+// that fill the SMs. Which one wins depends on N, the segment
 // lengths and the tree depths, so it is measured: each candidate runs the
 // same trial mutation on copies of the caller's particles, timed with CUDA
 // events on the launching stream. A NUTS result does not depend on the slot
