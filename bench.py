@@ -41,7 +41,9 @@ UNIT = "evals/s"
 #        each) per bin, the delay term in FP32 per detector.
 # split: FP32 phase, 8 split products per bin shared by 3 detectors + ~15
 #        FLOP per detector -> 51 FLOP, total 96 FP32 FLOP.
-# fp64: all eight terms in FP64 FMA, carrier by sincospi (~30 FMA), moments in FP64.
+# fp64: the phase (eight terms shared by 3 detectors, the delay) in FP64 FMA;
+#        carrier, data product and moments in 64-bit fixed point on the integer
+#        pipe (csrc/fixed.cuh): IMAD multiply-adds.
 # These estimates stand in only while no instruction counts of the current
 # kernel sources are recorded (COUNTED below).
 def work(precision, n_det=3):
@@ -53,10 +55,16 @@ def work(precision, n_det=3):
         return {"pipe": "fp64", "flop": 2.0 * 4.0 / n_det, "fp32_flop": 4.0 * 13.5 / n_det + delay32 + 45.0}
     if precision == "split":
         return {"pipe": "fp32", "flop": phase32 + 45.0, "fp32_flop": phase32 + 45.0}
-    return {"pipe": "fp64", "flop": poly64 + 2.0 + 60.0 + 45.0, "fp32_flop": 0.0}
+    return {"pipe": "fp64", "flop": poly64 + 2.0, "fp32_flop": 0.0}
 
 
 WORK = {p: work(p) for p in ("mixed", "split", "fp64")}
+# 32 x 32 + 64 bit multiply-adds and high products of the FP64 path's fixed-point
+# bins per active (bin, detector), from the source: sine and cosine of the rest
+# 11, rotations 24, nine basis moments 54, the plain one 4. They take the integer
+# multiply pipe, which is the busier one (57 % on the 259585-bin segment, the FP64
+# pipe 32 %); its rate is not probed, so no fraction of a peak is given.
+IMAD = {"fp64": 93.0}
 
 
 # Counter-derived work and traffic, valid only for the kernel sources they
@@ -64,33 +72,36 @@ WORK = {p: work(p) for p in ("mixed", "split", "fp64")}
 # above and traffic null). From one ncu launch each (`--mode nuts_launch
 # --ensemble late` for the NUTS kernel on the 11-D workload, `--mode
 # loglike_launch` with the tuned `--split` for the likelihood kernels):
-# FP64 FLOP = 2 DFMA + DADD + DMUL and FP32 FLOP = 2 FFMA + FADD + FMUL thread
-# instructions (smsp__sass_thread_inst_executed_op_*_pred_on.sum) per active
-# (bin, detector), and DRAM bytes read + written per launch.
+# FP64 FLOP = 2 DFMA + DADD + DMUL and FP32 FLOP = 2 FFMA + FADD + FMUL + 2 (2
+# FFMA2 + FADD2 + FMUL2) thread instructions (the last three packed;
+# smsp__sass_thread_inst_executed_op_*_pred_on.sum) per active (bin, detector),
+# and DRAM bytes read + written per launch.
 # Each kernel's counts are keyed to the device-code files its instructions
 # come from (context.cuh, the host-side context, is not among them).
-COUNTED_SOURCES = {"nuts": ["nuts_kernel.cuh", "sweep.cuh", "physics.cuh", "common.cuh", "dfloat.cuh"],
-                   "loglike": ["loglike_kernel.cuh", "bulk.cuh", "sweep.cuh", "physics.cuh",
+COUNTED_SOURCES = {"nuts": ["nuts_kernel.cuh", "sweep.cuh", "fixed.cuh", "physics.cuh", "common.cuh", "dfloat.cuh"],
+                   "loglike": ["loglike_kernel.cuh", "bulk.cuh", "sweep.cuh", "fixed.cuh", "physics.cuh",
                                "common.cuh", "dfloat.cuh"]}
-COUNTED = {"sources_sha256_16": {"nuts": "4c9bc0a722a82040", "loglike": "43066a7c70b78fc5"},
-           "nuts": {"mixed": {"fp64": 2.9620, "fp32": 107.01},
-                    "split": {"fp64": 0.2756, "fp32": 126.67},
-                    "fp64": {"fp64": 110.50, "fp32": 0.0152}},
+COUNTED = {"sources_sha256_16": {"nuts": "aa9ac21577eb2062", "loglike": "1475e786934fba37"},
+           "nuts": {"mixed": {"fp64": 2.9600, "fp32": 113.01},
+                    "split": {"fp64": 0.2736, "fp32": 132.68},
+                    "fp64": {"fp64": 15.413, "fp32": 0.0339}},
            # the likelihood kernels, one call each with the tuner's choice for
            # that shape: 2048 vectors of the 11-D workload (1 warp per vector),
-           # 8192 vectors of the 259585-bin segment (mixed and split: the staged
-           # kernel; FP64: 4 warps per vector)
-           "loglike": {"bbh11": {"mixed": {"fp64": 2.8057, "fp32": 88.321}},
-                       "bns": {"mixed": {"fp64": 2.6686, "fp32": 81.405},
-                               "split": {"fp64": 0.0019, "fp32": 101.07},
-                               "fp64": {"fp64": 90.365, "fp32": 0.0}}},
-           "traffic": {"mixed": 3830016, "split": 3913984, "fp64": 4599040},
-           # the same captures: FP64 pipe busy, warps active and issue active
+           # 8192 vectors of the 259585-bin segment (mixed and split: 8 warps
+           # per vector; FP64: 4)
+           "loglike": {"bbh11": {"mixed": {"fp64": 2.9158, "fp32": 94.454},
+                                 "fp64": {"fp64": 13.417, "fp32": 0.0310}},
+                       "bns": {"mixed": {"fp64": 2.6691, "fp32": 87.406},
+                               "split": {"fp64": 0.0020, "fp32": 107.07},
+                               "fp64": {"fp64": 7.5000, "fp32": 0.0}}},
+           "traffic": {"mixed": 794880, "split": 660992, "fp64": 915200},
+           # the same captures: FP64 pipe, warps and issue active
            # (sm__inst_executed_pipe_fp64, sm__warps_active,
-           # smsp__issue_active; % of peak sustained active)
-           "util": {"mixed": {"fp64_pipe": 34.4, "warps_active": 10.7, "issue_active": 37.0},
-                    "split": {"fp64_pipe": 16.6, "warps_active": 10.7, "issue_active": 40.2},
-                    "fp64": {"fp64_pipe": 86.0, "warps_active": 11.0, "issue_active": 8.0}}}
+           # smsp__issue_active; % of peak sustained active) and the integer
+           # multiply pipe (sm__pipe_fmaheavy_cycles_active, % of elapsed)
+           "util": {"mixed": {"fp64_pipe": 36.9, "warps_active": 12.5, "issue_active": 31.1, "imad_pipe": 19.4},
+                    "split": {"fp64_pipe": 12.3, "warps_active": 12.5, "issue_active": 35.9, "imad_pipe": 24.2},
+                    "fp64": {"fp64_pipe": 46.0, "warps_active": 10.7, "issue_active": 28.0, "imad_pipe": 29.0}}}
 
 
 def _sources_hash(kernel="nuts"):
@@ -127,9 +138,12 @@ def _util(precision):
     return COUNTED["util"].get(precision)
 
 
-def binding_pipe(f64, f32, p64, p32):
-    """(pipe, FLOP per unit, peak) of the pipe that bounds a kernel doing f64 FP64 and f32 FP32 FLOP per unit:
-    the one whose work takes longer at its peak (the two pipes issue concurrently)."""
+def binding_pipe(precision, f64, f32, p64, p32):
+    """(pipe, operations per unit, peak) of the pipe that bounds a kernel doing f64 FP64 and f32 FP32 FLOP per unit:
+    the one whose work takes longer at its peak (the two pipes issue concurrently). FP64 path: the integer
+    multiply-adds, no peak."""
+    if precision in IMAD:
+        return "imad", IMAD[precision], None
     if p32 and f32 / p32 > f64 / p64:
         return "fp32", f32, p32
     return "fp64", f64, p64
@@ -322,11 +336,15 @@ def main_loglike(args):
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1) / reps
             f64c, f32c, fsrc = counted("loglike", prec, w.name)
-            pipe, flop, peak = binding_pipe(f64c, f32c, peaks[1], peaks[0])
+            pipe, flop, peak = binding_pipe(prec, f64c, f32c, peaks[1], peaks[0])
+            if pipe == "imad":
+                fsrc = "multiply-adds counted in the source"
             tfl = n * act * flop / (ms * 1e-3) / 1e12
+            f64_tfl = n * act * f64c / (ms * 1e-3) / 1e12
             row[prec] = {"evals_per_s": n / (ms * 1e-3), "ms_per_call": ms, "pipe": pipe,
                          "flop_per_active_bin_det": flop, "flop_source": fsrc,
-                         "achieved_tflops": tfl, "frac": tfl / peak,
+                         "achieved_tflops": tfl, "frac": tfl / peak if peak else None,
+                         "fp64_frac": f64_tfl / peaks[1],
                          "warps_per_vector_tuned": ctx.loglike_split(n, prec)}
         out["sets"][name] = row
     # oracle on 64 vectors of the ball set, and the mixed path's error against it
@@ -575,7 +593,8 @@ def main_batch(args):
     n_ev = len(ws) * args.steps * world
     if rank == 0:
         f64c, f32c, _ = counted("nuts", args.precision)
-        wk = {"flop": f32c if args.precision == "split" else f64c}  # the pipe that binds on the 11-D workload
+        # the pipe that binds on the 11-D workload (FP64 path: of floating-point work)
+        wk = {"flop": f32c if args.precision == "split" else f64c}
         out = {"metric": METRIC, "value": total / (t_max * 1e-3), "unit": UNIT, "n_gpus": world,
                "steps": args.steps, "warmup": args.warmup, "ms_per_step": t_max / args.steps,
                "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
@@ -716,18 +735,21 @@ def main():
     lib().sharpy_probe_peaks(local, peaks)
     fp32_peak, fp64_peak = peaks[0], peaks[1]
     f64c, f32c, fsrc = counted("nuts", args.precision)
-    pipe, flop, peak = binding_pipe(f64c, f32c, fp64_peak, fp32_peak)
+    pipe, flop, peak = binding_pipe(args.precision, f64c, f32c, fp64_peak, fp32_peak)
+    if pipe == "imad":
+        fsrc = "multiply-adds counted in the source"
     secs = nuts_ms * 1e-3
     ach = bins * flop / secs / 1e12
     fp64_ach, fp32_ach = bins * f64c / secs / 1e12, bins * f32c / secs / 1e12
     kname = {"mixed": "MIXED", "split": "MIXED_SPLIT", "fp64": "FP64"}[args.precision]
     roofline = {"bound": "alu", "kernel": f"nuts_kernel<{kname},{w.n_det}>", "achieved": ach, "peak": peak,
-                "unit": "TFLOP/s", "frac": ach / peak if peak else None,
+                "unit": "TFLOP/s" if peak else "T multiply-adds/s (64-bit, integer pipe)",
+                "frac": ach / peak if peak else None,
                 "traffic": _traffic(args.precision) if w.name == "bbh11" else None,
                 "traffic_unit": "bytes per NUTS launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
                 "pipe": pipe, "flop_per_active_bin_det": flop, "flop_source": fsrc,
                 "fp64_flop_per_active_bin_det": f64c, "fp32_flop_per_active_bin_det": f32c,
-                "peak_source": f"measured {pipe.upper()} FMA probe on this GPU (sharpy_probe_peaks)",
+                "peak_source": f"measured {pipe.upper()} FMA probe on this GPU (sharpy_probe_peaks)" if peak else None,
                 "fp64_achieved": fp64_ach, "fp64_frac": fp64_ach / fp64_peak if fp64_peak else None,
                 "fp32_achieved": fp32_ach, "fp32_peak": fp32_peak,
                 "fp32_frac": fp32_ach / fp32_peak if fp32_peak else None, "fp64_peak": fp64_peak,
