@@ -482,3 +482,34 @@ def test_loglike_fp64_tuner_choices():
             lf, gf = ctx.loglike_grad(th, "fp64")
             assert torch.equal(lf, l) and torch.equal(gf, g), (n, split)
         ctx.set_loglike_split(0)
+
+
+@pytest.mark.parametrize("n_bins", [33, 700, 65536 + 17])
+def test_loglike_two_detectors(n_bins):
+    """Two detectors have their own branches in the sweeps (delays in one pair, no odd one): the three paths against
+    the oracle within the workloads' bounds, ln L alone and with its gradient, every choice of warps per vector the
+    same bits, the staged kernel of a long segment among them."""
+    G.require_gpu()
+    w = inputs.bbh11() if n_bins < 65536 else inputs.bns()
+    w.n_det, w.n_bins = 2, n_bins
+    ev, ctx, th_inj, _ = G.event_pair(w, seed=1)
+    th = np.vstack([inputs.prior_draws(w, 5, 51), inputs.ball(w, th_inj, 6, 52)])
+    ref_l, ref_g = oracle.loglike(helpers.oracle_model(w), ev, th)
+    wid = G.width(w)
+    norm = np.linalg.norm(ref_g * wid, axis=1)
+    for prec, ltol, gtol, floor in (("mixed", 1e-2 if n_bins > 65536 else 1e-3, 1e-4, 1e-3),
+                                    ("split", 1e-2 if n_bins > 65536 else 1e-3, 1e-4, 1e-3),
+                                    ("fp64", 1e-7, 1e-8, 1e-6)):
+        out = []
+        for split in (1, 2, 4, 8, 16):
+            ctx.set_loglike_split(split)
+            l, g = ctx.loglike_grad(G.to_dev(th), prec)
+            l0, _ = ctx.loglike_grad(G.to_dev(th), prec, grad=False)
+            out.append((l, g, l0))
+        ctx.set_loglike_split(0)
+        assert all(torch.equal(a, b) for o in out for a, b in zip(o, out[0])), prec
+        for x in (out[0][0], out[0][2]):
+            assert np.all(np.abs(x.cpu().numpy() - ref_l) <= ltol + 1e-10 * np.abs(ref_l)), prec
+        err = np.linalg.norm((out[0][1].cpu().numpy() - ref_g) * wid, axis=1)
+        assert np.all(err <= np.maximum(gtol * norm, floor)), (prec, err / norm)
+    assert ctx.status() == 0
