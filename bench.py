@@ -81,27 +81,27 @@ IMAD = {"fp64": 93.0}
 COUNTED_SOURCES = {"nuts": ["nuts_kernel.cuh", "sweep.cuh", "fixed.cuh", "physics.cuh", "common.cuh", "dfloat.cuh"],
                    "loglike": ["loglike_kernel.cuh", "bulk.cuh", "sweep.cuh", "fixed.cuh", "physics.cuh",
                                "common.cuh", "dfloat.cuh"]}
-COUNTED = {"sources_sha256_16": {"nuts": "c07fd72aa793fdbf", "loglike": "f2c13c20c2d51332"},
+COUNTED = {"sources_sha256_16": {"nuts": "aa9ac21577eb2062", "loglike": "1475e786934fba37"},
            "nuts": {"mixed": {"fp64": 2.9600, "fp32": 113.01},
                     "split": {"fp64": 0.2736, "fp32": 132.68},
                     "fp64": {"fp64": 15.413, "fp32": 0.0339}},
            # the likelihood kernels, one call each with the tuner's choice for
            # that shape: 2048 vectors of the 11-D workload (1 warp per vector),
            # 8192 vectors of the 259585-bin segment (mixed and split: 8 warps
-           # per vector; FP64: 2)
+           # per vector; FP64: 4)
            "loglike": {"bbh11": {"mixed": {"fp64": 2.9158, "fp32": 94.454},
                                  "fp64": {"fp64": 13.417, "fp32": 0.0310}},
                        "bns": {"mixed": {"fp64": 2.6691, "fp32": 87.406},
                                "split": {"fp64": 0.0020, "fp32": 107.07},
                                "fp64": {"fp64": 7.5000, "fp32": 0.0}}},
-           "traffic": {"mixed": 753664, "split": 660736, "fp64": 804352},
+           "traffic": {"mixed": 794880, "split": 660992, "fp64": 915200},
            # the same captures: FP64 pipe, warps and issue active
            # (sm__inst_executed_pipe_fp64, sm__warps_active,
            # smsp__issue_active; % of peak sustained active) and the integer
            # multiply pipe (sm__pipe_fmaheavy_cycles_active, % of elapsed)
            "util": {"mixed": {"fp64_pipe": 36.9, "warps_active": 12.5, "issue_active": 31.1, "imad_pipe": 19.4},
                     "split": {"fp64_pipe": 12.3, "warps_active": 12.5, "issue_active": 35.9, "imad_pipe": 24.2},
-                    "fp64": {"fp64_pipe": 45.5, "warps_active": 10.7, "issue_active": 27.7, "imad_pipe": 29.0}}}
+                    "fp64": {"fp64_pipe": 46.0, "warps_active": 10.7, "issue_active": 28.0, "imad_pipe": 29.0}}}
 
 
 def _sources_hash(kernel="nuts"):
