@@ -160,13 +160,12 @@ void sharpy_destroy(sharpy_ctx* ctx);
 int sharpy_set_data(sharpy_ctx* ctx, int n_det, int64_t n_bins, double f_min, double df,
                     const double* d_re_im, const double* psd, const sharpy_detector* det);
 
-/* Which arithmetic the FP64 path sums the staged event's bins in for a vector
-   whose last active bin (f_k <= f_ISCO) is last_bin: 1, 64-bit fixed point; 0,
-   FP64 (the sums would lose bits against FP64 there, because the data hold much
-   larger values just past that bin, or values that no scale fits before it, or
-   because nothing precedes it: the first 32 bins). A negative code on errors.
-   Synchronises with the default stream. */
-int sharpy_fixed_point_at(sharpy_ctx* ctx, int64_t last_bin);
+/* Which arithmetic the FP64 path sums the staged event's bins in: vectors
+   whose last active bin (f_k <= f_ISCO) is at least *bin in 64-bit fixed point,
+   the others in FP64 (their sums would lose bits against FP64 where the data
+   hold a much larger value further on). *bin = n_bins: all in FP64. Synchronises
+   with the default stream. */
+int sharpy_fixed_point_from(sharpy_ctx* ctx, int64_t* bin);
 
 /* Prior draws (Philox4x32-10, purpose 1, counter (particle, ctr, 1, dim)). theta: [N][D] device. */
 int sharpy_prior_sample(sharpy_ctx* ctx, int64_t n, double* theta, uint64_t key, uint64_t ctr,

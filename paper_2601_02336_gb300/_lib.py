@@ -66,7 +66,7 @@ _SIGS = {
     "sharpy_destroy": (None, [_CTX]),
     "sharpy_set_data": (C.c_int, [_CTX, C.c_int, C.c_int64, C.c_double, C.c_double, _VP, _VP,
                                   C.POINTER(Detector)]),
-    "sharpy_fixed_point_at": (C.c_int, [_CTX, C.c_int64]),
+    "sharpy_fixed_point_from": (C.c_int, [_CTX, C.POINTER(C.c_int64)]),
     "sharpy_prior_sample": (C.c_int, [_CTX, C.c_int64, _VP, C.c_uint64, C.c_uint64, _VP]),
     "sharpy_prior_logpdf_grad": (C.c_int, [_CTX, C.c_int64, _VP, _VP, _VP, _VP]),
     "sharpy_loglike_grad": (C.c_int, [_CTX, C.c_int64, _VP, _VP, _VP, C.c_int, _VP]),

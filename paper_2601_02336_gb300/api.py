@@ -113,12 +113,12 @@ class Context:
                                     dets), "sharpy_set_data")
         self.n_det, self.n_bins = n_det, n_bins
 
-    def fixed_point_at(self, last_bin):
-        """Whether the FP64 path sums a vector whose last active bin is last_bin in 64-bit fixed point (else FP64)."""
-        rc = lib().sharpy_fixed_point_at(self._h, int(last_bin))
-        if rc < 0:
-            check(rc, "sharpy_fixed_point_at")
-        return rc == 1
+    def fixed_point_from(self):
+        """The FP64 path sums vectors whose last active bin is at least this in 64-bit fixed point, the others in
+        FP64 (n_bins: all of them)."""
+        b = C.c_int64()
+        check(lib().sharpy_fixed_point_from(self._h, C.byref(b)), "sharpy_fixed_point_from")
+        return b.value
 
     # ---------------------------------------------------------- likelihood
     def loglike_grad(self, theta, precision="mixed", grad=True, out=None):

@@ -93,8 +93,8 @@ struct DevEvent {
   const float4* tile_mixed;  // tiles of the mixed and the split sweep, whole blocks of kStageBins
   const float4* tile_split;
   const int4* tile_fix;      // the FP64 path's bins in fixed point (fixed.cuh), or null: the FP64 sweep
-  const FixBlock* fix_block; // their scales and which sweeps they serve, per block of 256 bins
-  const int* fix_from;       // they serve every sweep whose last active bin is at least this
+  const int* fix_from;       // sweeps whose last active bin lies below take the FP64 sweep (read by the kernels: it goes with the tables)
+  const FixBlock* fix_block; // their scales, per block of 256 bins
   const int4* fix_trig;      // the carrier's table
   const double* pref;        // [n_det][K] prefix sums of w f^-7/3
   const double* p1;          // [n_det][kNBasis][K] prefix sums of w f^-7/3 B_m (Fisher), or null

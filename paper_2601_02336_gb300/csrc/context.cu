@@ -48,50 +48,45 @@ struct FixTables {
   int4* tile;
   FixBlock* block;
   double *sq, *need;   // [kFixDet * kNMom][blocks]
+  int* from;           // [blocks], then the event's fix_from
   unsigned int* done;  // blocks that have written these; zero between launches
-  int* from;           // the last block's `from` that is not zero (DevEvent::fix_from)
 };
 __device__ __forceinline__ uint32_t fix_abs_hi(double x) {  // |x|'s high word, zero for zero only
   return ((uint32_t)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0);
 }
 __device__ __forceinline__ double fix_pow2(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
-// The rule over all blocks, on the CTA that comes last: a warp a moment in turn,
+// fix_from over all blocks, on the CTA that comes last: a warp a moment in turn,
 // lanes over the blocks; an exclusive prefix sum of the blocks' squares against
-// what each needs before it.
+// what each needs before it. Past the last block that fails, or what the blocks
+// ask for themselves.
 __device__ void fix_from_all(int n_det, int blocks, const FixTables& fix) {
-  __shared__ int misfit_s;  // the first block without scales; what lies past it is not read
   __shared__ int from_s;
   const int lane = threadIdx.x & 31;
-  if (threadIdx.x == 0) misfit_s = blocks, from_s = __ldcg(&fix.block[0].from);
+  if (threadIdx.x == 0) from_s = 0;
   __syncthreads();
-  for (int g = threadIdx.x; g < blocks; g += blockDim.x)
-    if (__ldcg(&fix.block[g].from) == kFixNever) atomicMin(&misfit_s, g);
-  __syncthreads();
-  const int misfit = misfit_s;
-  for (int g = misfit + threadIdx.x; g < blocks; g += blockDim.x) fix.block[g].from = kFixNever;
+  int from = 0;
+  for (int g = threadIdx.x; g < blocks; g += blockDim.x) from = max(from, __ldcg(fix.from + g));
   for (int n = threadIdx.x >> 5; n < n_det * kNMom; n += blockDim.x >> 5) {
     const double *sqs = fix.sq + (int64_t)n * blocks, *needs = fix.need + (int64_t)n * blocks;
     double before = 0.0;
-    for (int g0 = 0; g0 < misfit; g0 += 32) {
+    for (int g0 = 0; g0 < blocks; g0 += 32) {
       const int g = g0 + lane;
-      double incl = g < misfit ? __ldcg(sqs + g) : 0.0;
-      const double need = g < misfit ? __ldcg(needs + g) : 0.0;
+      double incl = g < blocks ? __ldcg(sqs + g) : 0.0;
+      const double need = g < blocks ? __ldcg(needs + g) : 0.0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const double x = __shfl_up_sync(0xffffffffu, incl, o);
         if (lane >= o) incl += x;
       }
       const double excl = __shfl_up_sync(0xffffffffu, incl, 1);
-      if (g < misfit && !(need <= before + (lane ? excl : 0.0))) {
-        atomicMax(&fix.block[g].from, (g + 1) * kFixBins);
-        atomicMax(&from_s, (g + 1) * kFixBins);
-      }
+      if (!(need <= before + (lane ? excl : 0.0))) from = max(from, (g + 1) * kFixBins);
       before += __shfl_sync(0xffffffffu, incl, 31);
     }
   }
+  atomicMax(&from_s, from);
   __syncthreads();
-  if (threadIdx.x == 0) *fix.from = misfit < blocks ? kFixNever : from_s;
+  if (threadIdx.x == 0) fix.from[blocks] = from_s;
 }
 
 static_assert(kFixBins == kStageBins, "one block size");
@@ -171,7 +166,7 @@ __global__ void __launch_bounds__(kStageBins)
   for (int j = 0; j < kNBasis; ++j) eb[j] = expo(kFixDet + j);
   eb[kNBasis] = -1;
   if (!fits) {
-    if (threadIdx.x == 0) fix.block[blockIdx.x].from = kFixNever;
+    if (threadIdx.x == 0) fix.from[blockIdx.x] = kFixNever;
   } else {
     // products p < 4 sqrt(2) of this tile, rounded outwards by the factor
     {
@@ -238,7 +233,7 @@ __global__ void __launch_bounds__(kStageBins)
       }
       __syncwarp();
       last = __reduce_max_sync(0xffffffffu, last);
-      if (lane == 0) fc.from = blockIdx.x == 0 ? kTileBins * (last + 1) : 0;
+      if (lane == 0) fix.from[blockIdx.x] = blockIdx.x == 0 ? kTileBins * (last + 1) : 0;
     }
     __syncthreads();
     int4* t = fix.tile + tile * (kFixQuads * kTileBins) + lane;
@@ -302,8 +297,8 @@ static cudaError_t build_tables(sharpy_ctx* c, int64_t blocks) {
   float4* split = c->d_tile + blocks * (stage_bytes(false) / 16);
   const size_t tiles = (size_t)blocks * kStageBins * kFixQuads, rule = (size_t)blocks * kFixDet * kNMom;
   if (!c->d_fix && ev.n_bins <= kFixMaxBins && ev.n_det <= kFixDet) {
-    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig + 1) * sizeof(int4) + (size_t)blocks * sizeof(FixBlock) +
-                                  2 * rule * sizeof(double)) != cudaSuccess) {
+    if (cudaMalloc(&c->d_fix, (tiles + kFixTrig + 1) * sizeof(int4) + (size_t)blocks * (sizeof(FixBlock) + sizeof(int)) +
+                                  2 * rule * sizeof(double) + sizeof(int)) != cudaSuccess) {
       c->d_fix = nullptr;
       (void)cudaGetLastError();
     } else {
@@ -315,10 +310,10 @@ static cudaError_t build_tables(sharpy_ctx* c, int64_t blocks) {
   if (c->d_fix) {
     fix.tile = c->d_fix;
     fix.done = reinterpret_cast<unsigned int*>(c->d_fix + tiles + kFixTrig);
-    fix.from = reinterpret_cast<int*>(fix.done + 1);
     fix.block = reinterpret_cast<FixBlock*>(c->d_fix + tiles + kFixTrig + 1);
     fix.sq = reinterpret_cast<double*>(fix.block + blocks);
     fix.need = fix.sq + rule;
+    fix.from = reinterpret_cast<int*>(fix.need + rule);
   }
   event_tables_kernel<<<(unsigned)blocks, kStageBins>>>(ev, c->d_tile, split, fix);
   const cudaError_t e = cudaGetLastError();
@@ -327,8 +322,8 @@ static cudaError_t build_tables(sharpy_ctx* c, int64_t blocks) {
   ev.tile_split = split;
   if (c->d_fix) {
     ev.tile_fix = fix.tile;
+    ev.fix_from = fix.from + blocks;
     ev.fix_block = fix.block;
-    ev.fix_from = fix.from;
     ev.fix_trig = c->d_fix + tiles;
   }
   return cudaSuccess;
@@ -580,14 +575,15 @@ int sharpy_set_data(sharpy_ctx* c, int n_det, int64_t n_bins, double f_min, doub
   return SHARPY_OK;
 }
 
-int sharpy_fixed_point_at(sharpy_ctx* c, int64_t last_bin) {
+int sharpy_fixed_point_from(sharpy_ctx* c, int64_t* bin) {
   int rc = check_ctx(c, true);
   if (rc) return rc;
-  if (c->model.model != SHARPY_MODEL_TAYLORF2 || last_bin < 0 || last_bin >= c->ev.n_bins) return SHARPY_EINVAL;
-  if (!c->ev.tile_fix) return 0;
-  int from = 0;
-  SHARPY_CUDA_TRY(cudaMemcpy(&from, &c->ev.fix_block[last_bin / kFixBins].from, sizeof(int), cudaMemcpyDeviceToHost));
-  return last_bin >= from ? 1 : 0;
+  if (!bin) return SHARPY_EINVAL;
+  if (c->model.model != SHARPY_MODEL_TAYLORF2) return SHARPY_EINVAL;
+  int from = kFixNever;
+  if (c->ev.tile_fix) SHARPY_CUDA_TRY(cudaMemcpy(&from, c->ev.fix_from, sizeof(int), cudaMemcpyDeviceToHost));
+  *bin = from < c->ev.n_bins ? from : c->ev.n_bins;
+  return SHARPY_OK;
 }
 
 int sharpy_reset_evidence(sharpy_ctx* c, sharpy_stream stream) {

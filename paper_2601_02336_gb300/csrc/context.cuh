@@ -31,7 +31,7 @@ struct sharpy_ctx {
   double* d_b64 = nullptr;
   double2* d_e64 = nullptr;
   float4* d_tile = nullptr;  // the mixed sweep's tiles, then the split sweep's
-  int4* d_fix = nullptr;     // the FP64 path's fixed-point tiles, the carrier table, the blocks' scales and rule
+  int4* d_fix = nullptr;     // the FP64 path's fixed-point tiles, the carrier table, the blocks' scales and rule, fix_from
   double* d_pref = nullptr;
   // status word and evidence accumulator (device)
   int* d_status = nullptr;

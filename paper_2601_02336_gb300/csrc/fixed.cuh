@@ -34,12 +34,11 @@
 // events (noise, signal, both; 10 or 20 Hz; one bin up to 2^12 times too large;
 // host emulation against 128 bits, 12 000 sweeps) the moments' errors are then
 // 0.5 times FP64's in the median and 2.7 times at most (mean of the ten); past
-// the line the ratio grows with it, without bound. Sweeps that end in a block
-// before its bin `from` take the FP64 sweep: in the first block up to the last
-// tile that fails, the first tile at least (nothing precedes its bins); in a later
-// one all of them if one fails; from a block on that no scale fits, all. Noise
-// from 20 Hz has no failure but the first tile; noise from 10 Hz, where the data
-// rise by 2^5 within a block, has some in the first block.
+// the line the ratio grows with it, without bound. Sweeps that end before the bin fix_from of the event (the last
+// failure, at least the first tile, whose bins nothing precedes) take the FP64
+// sweep: noise from 20 Hz has no other failure, noise from 10 Hz, where the data
+// rise by 2^5 within a block, some in the first block. Data that no scale fits
+// keep the FP64 sweep throughout.
 #pragma once
 #include <cstdint>
 #include <cstring>
@@ -54,15 +53,13 @@ constexpr int kFixDet = 3;                // detectors at most
 constexpr int kFixQuads = kNBasis + kFixDet;
 constexpr int kFixBins = 256;             // bins that share their scales: 8 lane iterations
 constexpr int64_t kFixMaxBins = 1 << 24;  // 3.2 GB of tiles; more bins keep the FP64 sweep
-constexpr int kFixNever = 0x7fffffff;     // `from` past values that no scale fits
+constexpr int kFixNever = 0x7fffffff;     // fix_from of data that no scale fits
 constexpr int kFixTrig = 1024;            // points of the carrier table, {cos h, l, sin h, l} to 2^-62
 
-// A block's scales, moment (a, j) = scale[a * kNMom + j] x integer sum, and the
-// sweeps that it serves.
+// A block's scales: moment (a, j) = scale[a * kNMom + j] x integer sum.
 struct FixBlock {
   double scale[kFixDet * kNMom];
-  int one;   // high limb of the basis value 1
-  int from;  // sweeps that end in this block before bin `from` take the FP64 sweep
+  int one;  // high limb of the basis value 1
 };
 
 // Whether a sweep that ends in tile t of a block fails: `unit` of the block's

@@ -632,17 +632,10 @@ __device__ bool fp64_stream(const DevEvent& ev, const SweepCoef& sc, int s, doub
 }
 
 // One stream of the FP64 path, in the arithmetic that the event's data allow
-// for a sweep of this length (fixed.cuh). fix_from, from which on all ends are
-// served, is one address for all sweeps; a shorter sweep looks at its block, out
-// of line: with each sweep reading its own block a mutation took 1 to 4 % longer
-// (the read's latency is in every tick's chain), inlined 1 %, so 0.3 %.
-static __device__ __noinline__ bool fix_serves(const FixBlock* blocks, int kisco) {
-  return kisco >= blocks[max(kisco, 0) / kFixBins].from;
-}
+// for a sweep of this length (fixed.cuh).
 template <bool GRAD, int NDET>
 __device__ bool wide_stream(const DevEvent& ev, const SweepCoef& sc, int s, double* v_out) {
-  const bool fixed = ev.tile_fix && (sc.kisco >= *ev.fix_from || fix_serves(ev.fix_block, sc.kisco));
-  return fixed ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
+  return ev.tile_fix && sc.kisco >= *ev.fix_from ? fixed_stream<GRAD, NDET>(ev, sc, s, v_out) : fp64_stream<GRAD, NDET>(ev, sc, s, v_out);
 }
 
 // FP64 moments of one particle on one warp; streams as in sweep_mixed (a
